@@ -235,8 +235,9 @@ wcsim_status wcsim_plane_set_reuse_forward(wcsim_plane* plane, int32_t enable);
  * Host-only. */
 wcsim_status wcsim_plane_set_forward(wcsim_plane* plane, int32_t fused);
 
-/* Rasterization tile of this plane (the autotuner's first choice, settable by hand):
- * depos_per_block depos per CTA of 256 threads, each rasterized by lanes_per_depo lanes.
+/* Rasterization tile of this plane (the autotuner's first choice, settable by hand; without
+ * either, each call takes one by its number of depos): depos_per_block depos per 256 threads,
+ * each rasterized by lanes_per_depo lanes.
  * Supported: (32, 8), (64, 8), (128, 8), (256, 8), (64, 16), (128, 16), (256, 16),
  * (64, 32), (128, 32), (256, 32); WCSIM_EINVAL otherwise.  Results are unchanged up to summation order.
  * Host-only. */
@@ -248,7 +249,7 @@ typedef struct {
     int32_t time_radix[8];     /* radices of the time-axis FFT plan, in pass order, 0-padded */
     int32_t rows_variant;      /* time-axis forward kernel: 0 direct loads, 1 bulk-staged */
     int32_t wire_variant;      /* wire pass: 0 one warp per time frequency, 1 block-level */
-    int32_t depos_per_block;   /* rasterization tile: depos per CTA, 32..256 */
+    int32_t depos_per_block;   /* rasterization tile: depos per 256 threads, 8..256 */
     int32_t candidates_timed;  /* configurations timed */
     float ms_rasterize, ms_rows, ms_wire;
     int32_t forward_fused;     /* forward variant kept (wcsim_plane_set_forward) */

@@ -105,8 +105,8 @@ struct wcsim_plane {
     wcsim_drift_params fwd_prm = {};
     bool wire_block = false;    // autotuned: use the block-level wire pass even if the warp one fits
     bool adj_block = false;     // use the block-level wire adjoint even if the warp one fits
-    int32_t kd = 32;            // rasterization tile: depos per CTA and lanes per depo (the
-    int32_t kg = 8;             // autotuner may change them)
+    int32_t kd = 0;             // rasterization tile set by hand or by the autotuner: depos per
+    int32_t kg = 0;             // 8 warps and lanes per depo (0: chosen per call, raster_tile)
     // forward with rasterization fused into the time-axis transform: depo binning scratch,
     // and the impact positions per wire-pass launch (the time-axis spectra of that many
     // impact positions are alive at a time)
@@ -196,8 +196,7 @@ RasterConsts make_consts(const wcsim_plane* pl)
     c.n_ticks = g.n_ticks;
     c.fluctuate = p.fluctuate;
     c.renorm = p.renormalize;
-    c.key0 = (uint32_t)p.seed;
-    c.key1 = (uint32_t)(p.seed >> 32);
+    c.keys.set((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
     c.plane_id = p.plane_id;
     c.depos_per_block = pl->kd;
     c.lanes_per_depo = pl->kg;
@@ -474,6 +473,9 @@ wcsim_status rasterize_group(wcsim_plane* pl, int k, const int32_t* idx, const w
     BatchEvents ev;
     ev.n = k;
     ev.block_start[0] = 0;
+    int64_t total = 0;
+    for (int i = 0; i < k; ++i) total += depos[idx[i]].n;
+    const RasterTile tile = raster_tile(c, total);
     for (int i = 0; i < k; ++i) {
         const wcsim_depos* dp = &depos[idx[i]];
         ev.d[i] = depo_arrays(dp);
@@ -481,9 +483,9 @@ wcsim_status rasterize_group(wcsim_plane* pl, int k, const int32_t* idx, const w
         const uint64_t seed = pl->prm.seed + (uint64_t)idx[i];     // per-event stream
         ev.key0[i] = (uint32_t)seed;
         ev.key1[i] = (uint32_t)(seed >> 32);
-        ev.block_start[i + 1] = ev.block_start[i] + rasterize_blocks(dp->n, c.depos_per_block);
+        ev.block_start[i + 1] = ev.block_start[i] + rasterize_blocks(dp->n, tile.depos_per_warp);
     }
-    cudaError_t e = launch_rasterize_batch(c, ev, pl->flags, s);
+    cudaError_t e = launch_rasterize_batch(c, ev, tile, pl->flags, s);
     return e ? cuda_fail(e, "batch rasterize launch") : WCSIM_OK;
 }
 
@@ -941,31 +943,33 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
         if (st) return st;
     }
     // one persistent rasterization over every event of the batch (a work queue of (event,
-    // depo block) items) when the planes share the rasterization tile and the kind of
-    // fluctuation draw; otherwise one launch per plane
+    // depo block) items) when the planes share the rasterization tile and the fluctuation mode;
+    // otherwise one launch per plane
     bool queue = true;
     const RasterConsts c0 = make_consts(planes[0]);
     for (int i = 1; i < n_events && queue; ++i) {
         const wcsim_plane* p = planes[i];
         queue = p->kd == planes[0]->kd && p->kg == planes[0]->kg &&
-                (p->prm.fluctuate == 2) == (c0.fluctuate == 2);
+                p->prm.fluctuate == c0.fluctuate;
     }
     if (queue) {
         QueueEvents q;
+        int64_t n_depos = 0;
+        for (int i = 0; i < n_events; ++i) n_depos += depos[i].n;
+        const RasterTile tile = raster_tile(c0, n_depos);
         q.n = n_events;
         q.block_start[0] = 0;
         for (int i = 0; i < n_events; ++i) {
             wcsim_plane* p = planes[i];
             q.c[i] = make_consts(p);
             const uint64_t seed = p->prm.seed + (uint64_t)i;         // per-event stream
-            q.c[i].key0 = (uint32_t)seed;
-            q.c[i].key1 = (uint32_t)(seed >> 32);
+            q.c[i].keys.set((uint32_t)seed, (uint32_t)(seed >> 32));
             q.d[i] = depo_arrays(&depos[i]);
             q.grid[i] = p->bgrid + (size_t)slot[i] * ev_grid_elems(p->dims);
             q.flags[i] = p->flags;
-            q.block_start[i + 1] = q.block_start[i] + rasterize_blocks(depos[i].n, c0.depos_per_block);
+            q.block_start[i + 1] = q.block_start[i] + rasterize_blocks(depos[i].n, tile.depos_per_warp);
         }
-        cudaError_t e = launch_rasterize_queue(q, planes[0]->queue, s);
+        cudaError_t e = launch_rasterize_queue(q, tile, planes[0]->queue, s);
         if (e) return cuda_fail(e, "batch rasterize launch");
     } else {
         for (int g = 0; g < n_groups; ++g) {
@@ -1014,20 +1018,28 @@ wcsim_status wcsim_plane_autotune(wcsim_plane* pl, const wcsim_depos* depos, voi
         return best;
     };
     wcsim_tune_report rep{};
-    // 1. rasterization tile: depos per CTA, lanes per depo
+    // 1. rasterization tile: depos per 8 warps, lanes per depo
     {
-        const int tiles[][2] = {{32, 8}, {64, 8}, {128, 8}, {256, 8}, {64, 16}, {128, 16},
-                                {256, 16}, {64, 32}, {128, 32}, {256, 32}};
+        const int tiles[][2] = {{0, 0}, {32, 8}, {64, 8}, {128, 8}, {256, 8}, {64, 16}, {128, 16},
+                                {256, 16}, {64, 32}, {128, 32}, {256, 32}};    // {0, 0}: the rule
         float best = 1e30f;
+        int keep_kd = 0, keep_kg = 0;
         for (const auto& t : tiles) {
             pl->kd = t[0];
             pl->kg = t[1];
             RasterConsts c = make_consts(pl);
             const float ms = time_it([&] { return launch_rasterize(c, depo_arrays(depos), pl->grid, pl->flags, s); });
-            if (ms < best) { best = ms; rep.depos_per_block = t[0]; rep.lanes_per_depo = t[1]; }
+            if (ms < best) {
+                const RasterTile rt = raster_tile(c, depos->n);
+                best = ms;
+                keep_kd = t[0];
+                keep_kg = t[1];
+                rep.depos_per_block = 8 * rt.depos_per_warp;
+                rep.lanes_per_depo = rt.lanes_per_depo;
+            }
         }
-        pl->kd = rep.depos_per_block;
-        pl->kg = rep.lanes_per_depo;
+        pl->kd = keep_kd;
+        pl->kg = keep_kg;
         rep.ms_rasterize = best;
         // a representative grid for the FFT stages
         if (!err) err = cudaMemsetAsync(pl->grid, 0, grid_bytes, s);

@@ -58,24 +58,73 @@ static __device__ __forceinline__ float window_mass(float frac, float hw, float 
     return span_mass(ua, ub, erfcf(fabsf(ua)), erfcf(fabsf(ub)));
 }
 
+// (float)x of a double, round to nearest even, by integer operations on its bits when the result
+// is a normal float (or x is +0); the conversion instruction, which runs on the FP64 pipe,
+// otherwise.  FP64 runs at 1/64 of the FP32 rate on this part, and a warp instruction costs the
+// same however many of its lanes are active: a bin decision taken with FP64 instructions
+// throughout held that pipe for 480 cycles per warp, which bounded the rasterizer when a warp
+// decides few depos.
+static __device__ __forceinline__ float double_to_float(double x)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t e = (uint32_t)(b >> 52) & 0x7ffu;
+    if (e - 897u < 253u) {                          // 2^-126 <= |x| < 2^127
+        const uint64_t m = (b & 0x7fffffffffffffffull) - (896ull << 52);
+        const uint32_t f = (uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1u)) >> 29);
+        return __uint_as_float(f | ((uint32_t)(b >> 32) & 0x80000000u));
+    }
+    return b == 0 ? 0.0f : __double2float_rn(x);
+}
+
+// floor(x) as an integer and frac = (float)(x - floor(x)), round to nearest even, by integer
+// operations for 1 <= x < 2^31 (every depo inside a grid but those of its first bin; x - floor(x)
+// is exact there): the fraction's bits, normalised, with the ones below the top 32 folded into
+// the lowest, round once in the integer conversion.  The FP64 operations themselves otherwise.
+static __device__ __forceinline__ bool floor_frac(double x, int64_t& i0i, float& frac)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t e = (uint32_t)(b >> 52) - 1023u; // sign bit set: far above 30
+    if (e < 31u) {
+        const uint64_t m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+        i0i = (int64_t)(m >> (52u - e));
+        const uint64_t f = m << (12u + e);          // x - floor(x) in units of 2^-64
+        const int lz = __clzll((long long)f);
+        if (lz >= 64) {
+            frac = 0.0f;
+            return true;
+        }
+        const uint64_t n = f << lz;
+        const uint32_t h = (uint32_t)(n >> 32) | ((uint32_t)n != 0u ? 1u : 0u);
+        frac = __uint2float_rn(h) * __uint_as_float((uint32_t)(95 - lz) << 23);   // 2^(-32 - lz)
+        return true;
+    }
+    if (!(fabs(x) < 1e12)) return false;
+    const double i0 = floor(x);
+    i0i = (int64_t)i0;
+    frac = __double2float_rn(__dsub_rn(x, i0));
+    return true;
+}
+
 // One axis of the bin decision.  Every operation is an explicitly rounded IEEE operation
 // (no contraction), so that the result is a function of the inputs alone.  The window edges
 // i0 + floor(frac -+ hw) are sums of whole numbers below 2^53, exact in FP64 and formed here
-// in 64-bit integers instead (FP64 runs at a small fraction of the FP32 rate on this part):
-// floor of a float is floorf, and clamping it to +-2^42 (far beyond |i0| < 10^12 and the grid)
-// changes no clipped edge.
+// in 64-bit integers instead: floor of a float is floorf, and clamping it to +-2^42 (far beyond
+// |i0| < 10^12 and the grid) changes no clipped edge.
 static __device__ __forceinline__ bool axis_window(double x, float hw, int64_t n, int32_t& lo,
                                             int32_t& hi, int64_t& i0i, float& frac)
 {
-    if (!(fabs(x) < 1e12)) return false;
-    const double i0 = floor(x);
-    frac = __double2float_rn(__dsub_rn(x, i0));
+    if (!floor_frac(x, i0i, frac)) return false;
     const float a = __fsub_rn(frac, hw);
     const float b = __fadd_rn(frac, hw);
     constexpr float kEdge = 4398046511104.0f;      // 2^42
-    i0i = (int64_t)i0;
-    int64_t l = i0i + (int64_t)fminf(fmaxf(floorf(a), -kEdge), kEdge);
-    int64_t h = i0i + (int64_t)fminf(fmaxf(floorf(b), -kEdge), kEdge);
+    int64_t l, h;
+    if (hw < 1e9f) {                               // both edges convert to 32-bit integers
+        l = i0i + (int32_t)floorf(a);
+        h = i0i + (int32_t)floorf(b);
+    } else {
+        l = i0i + (int64_t)fminf(fmaxf(floorf(a), -kEdge), kEdge);
+        h = i0i + (int64_t)fminf(fmaxf(floorf(b), -kEdge), kEdge);
+    }
     if (l < 0) l = 0;
     if (h > n - 1) h = n - 1;
     if (l > h) return false;
@@ -109,7 +158,7 @@ static __device__ __forceinline__ Decision decide(const RasterConsts& c, const D
         return r;
     }
     if (!(q > 0.0f)) return r;
-    const float td_f = __double2float_rn(td);
+    const float td_f = double_to_float(td);
     r.sp = __fsqrt_rn(__fmul_rn(c.two_dt, td_f));
     r.st = __fmul_rn(__fsqrt_rn(__fmul_rn(c.two_dl, td_f)), c.inv_v);
     const float hw_p = __fmul_rn(__fmul_rn(c.nsig, r.sp), c.inv_dp_f);

@@ -319,15 +319,8 @@ k_rows_r2c_fused(ConvDims d, FftPlan p, RasterConsts c, FusedBins b, float2* __r
             float v[4] = {wr * wt.x, wr * wt.y, wr * wt.z, wr * wt.w};
             if (c.fluctuate == 1) {
                 // normal approximation to Binomial(Q', mean / Q'); zero-mean bins stay zero
-                float z[4];
-                box_muller4(philox(make_uint4((uint32_t)q, (uint32_t)(row ? r1 : r0), s_id[h],
-                                              c.plane_id), c.key0, c.key1), z);
-                const float inv_q = s_invq[h];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float var = v[e] * (1.0f - v[e] * inv_q);
-                    v[e] = fmaxf(0.0f, fmaf(sqrt_fast(var), z[e], v[e]));
-                }
+                fluctuate4(philox_rounds<0>(make_uint4((uint32_t)q, (uint32_t)(row ? r1 : r0),
+                                                       s_id[h], c.plane_id), c.keys), s_invq[h], v);
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e)

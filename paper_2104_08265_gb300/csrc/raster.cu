@@ -2,14 +2,12 @@
 // (Sec. 2.1.1 "rasterization" and "scatter adding"; drift and diffusion as in Fig. 2;
 // fluctuation with a Box-Muller normal as in Sec. 4.3.1).
 //
-// Work split.  A block of 8 warps owns KD consecutive depos (32 by default; 64 or 128 when
-// the autotuner finds them faster; the adjoint uses 64).  Threads 0..KD-1 take the FP64 bin
-// decision of one depo each (one thread per depo: FP64 is scarce on this part, so it is
-// never evaluated redundantly by a whole warp) and park it in shared memory.  Each group of
-// 8 lanes then walks KD / 32 of the block's depos (the four groups of a warp work on four
-// depos side by side): its lanes compute one erfc per bin edge of the patch (rows and ticks
-// together), difference them into the per-bin 1D weights in shared memory and stride over
-// (row, 4-tick group) items.
+// Work split.  A warp owns a run of consecutive depos (4 to 32, chosen by the number of depos).
+// Its lanes take the bin decision of one depo each and park what the rasterization needs of it in
+// shared memory; then each group of 8 lanes takes the warp's depos one by one (the four groups of
+// a warp work on four depos side by side): its lanes compute one erfc per bin edge of the patch
+// (rows and ticks together), difference them into the per-bin 1D weights in shared memory and
+// stride over (row, 4-tick group) items.  Warps never wait for one another.
 // An item draws one Philox block for its four ticks when fluctuating (four Box-Muller
 // normals), forms Q' w_p w_t per bin and adds the four values into the grid with one
 // vector reduction.  The exact binomial fluctuation (an instance of its own) strides over
@@ -29,22 +27,23 @@
 namespace wcsim {
 namespace {
 
-constexpr int kWarps = 8;       // warps per block
-constexpr int kDepos = 64;      // depos per block
-constexpr int kWmax = 64;       // weights per axis held per patch tile
+constexpr int kRasterWarps = 4; // warps per block of the rasterizers
+constexpr int kWarps = 8;       // warps per block of the adjoint
+constexpr int kDepos = 64;      // depos per block of the adjoint
+constexpr int kWmax = 32;       // weights per axis held per patch tile
 
 // Exact binomial fluctuation of the bin (row r, tick k) with mean v: x ~ Binomial(N, p) with
 // N = rint(Q') whole electrons and p = v / Q', drawn by inversion at the 23-bit uniform of
 // word k mod 4 of the bin's Philox block (the block the normal approximation uses).  A bin
 // whose variance N p (1 - p) exceeds 65536, or N above 2^24, takes the normal
 // approximation instead.
-__device__ __forceinline__ float binomial_bin(const RasterConsts& c, const Decision& dd, int k,
+__device__ __forceinline__ float binomial_bin(const RasterConsts& c, float qatt, uint32_t id, int k,
                                               int64_t r, float v, float inv_q, const float* stirl)
 {
-    const uint4 x = philox(make_uint4((uint32_t)(k >> 2), (uint32_t)r, dd.id, c.plane_id),
-                           c.key0, c.key1);
+    const uint4 x = philox_rounds<0>(make_uint4((uint32_t)(k >> 2), (uint32_t)r, id, c.plane_id),
+                                     c.keys);
     const int e = k & 3;
-    const float n = rintf(dd.qatt);
+    const float n = rintf(qatt);
     const float p = fminf(1.0f, v * inv_q);
     if (n > 16777216.0f || n * p * (1.0f - p) > 65536.0f) {
         float z[4];
@@ -59,96 +58,253 @@ __device__ __forceinline__ float binomial_bin(const RasterConsts& c, const Decis
     return binomial_inverse(n, p, uniform23(w), stirl);
 }
 
-// The rasterization tiles (KD depos per CTA, G lanes per depo) the autotuner chooses from.
-// With G = 8 the four groups of a warp work on four depos side by side (a patch of ~17 rows x
-// 3 four-tick groups, ~47 items, fills six rounds of 8 lanes); with G = 32 a warp takes one
-// depo at a time (two rounds, but no groups diverging inside the warp).
-#define WCSIM_RASTER_TILES(X) X(32, 8) X(64, 8) X(128, 8) X(256, 8) X(64, 16) X(128, 16) \
-    X(256, 16) X(64, 32) X(128, 32) X(256, 32)
+// What the lanes of a group need of one depo, formed once by the lane that decides it.  Bin edge e
+// of the window (e bins above its first) lies at u = ((off + e) - frac) s, off the window's first
+// bin relative to the floor of the position (exact in FP32 below 2^24 bins).  A point (sigma == 0,
+// all weight in the window's one bin) has its edges far out on either side.
+//
+// Bin masses come in two forms.  In general they are differences of erfc at the edges.  Where the
+// bins are not wide against sigma, the mass about a bin's centre c (in units of sqrt(2) sigma,
+// half width s / 2) is
+//   1/2 (erf(c + s/2) - erf(c - s/2)) = erf(s/2) e^(-c^2) sum_k A_k / A_0 (c s)^(2k) / (2k)!,
+//   A_k = int_0^1 x^(2k) e^(-(s x / 2)^2) dx,
+// (the even part of e^(-2 c x) in the integral of e^(-(c + x)^2)): one exponential and ten terms,
+// all positive, per bin, with no cancellation, where the erfc form takes two edges and loses the
+// digits their difference cancels.  `series` marks a depo whose bins all have (c s)^2 <= 20 and
+// s <= 2.8 on both axes (sigma above about half a bin at 3 sigma), where ten terms and the
+// recurrence below leave less than 5e-8.
+// Instructions per four depos (960 x 6000 plane, warp counts): 400 with erfc, 170 with the series.
+constexpr int kTerms = 10;
+struct __align__(16) PatchDepo {
+    int32_t r_lo, nr, k_lo, nt;      // window; nr == 0: the depo adds nothing
+    float off_p, frac_p, s_p, qw;
+    float off_t, frac_t, s_t, inv_q;
+    float qatt;
+    uint32_t id;
+    int32_t series;
+    float pad;
+    float term[2][kTerms + 2];       // series_terms of the ticks and of the rows
+};
 
-// The depos [blk * KD, blk * KD + KD) of one event, by one CTA of kWarps warps, G lanes per
-// depo.  BIN: the exact binomial fluctuation (an instance of its own, so that the other
-// modes keep their registers).
-template <int KD, int G, bool BIN>
-__device__ __forceinline__ void rasterize_block(const RasterConsts& c, const DepoArrays& d,
-                                                float* __restrict__ grid, int* flags, int64_t blk)
+// (float)k, by the 32-bit conversion where it holds k.
+__device__ __forceinline__ float offset_float(int64_t k)
 {
-    static_assert(KD <= kWarps * 32, "one deciding thread per depo");
-    static_assert(G == 8 || G == 16 || G == 32, "lanes per depo");
-    constexpr int NG = kWarps * 32 / G;
-    __shared__ Decision s_dec[KD];
-    __shared__ float s_wp[NG][kWmax];
-    // tick weights of a tile laid out on 4-tick groups: slot p is tick 4 q_lo + p (zero
-    // outside the window), so that an item reads its four weights with one 16-byte load
-    __shared__ __align__(16) float s_wt[NG][kWmax + 8];
-    __shared__ float s_edge[NG][2 * (kWmax + 1)];        // row edges, then tick edges
-    __shared__ float s_stirl[BIN ? 16 : 1];              // the binomial's small-count table
-    if (BIN && threadIdx.x == 0) {
+    const int32_t k32 = (int32_t)k;
+    return (int64_t)k32 == k ? (float)k32 : (float)k;
+}
+
+__device__ __forceinline__ void edge_axis(float sigma, float bin, float frac, float& f, float& s)
+{
+    const bool point = !(sigma > 0.0f);
+    s = point ? 1e30f : bin / (1.41421356237309505f * sigma);
+    f = point ? 0.5f : frac;
+}
+
+// Series terms of one axis: term[0] = erf(s / 2), the mass of a bin about the mean, to which the
+// series comes down at c = 0, and term[k] = A_k / (A_0 (2k)!), with A_k by the downward recurrence
+// A_k = (e^(-h^2) + 2 h^2 A_(k+1)) / (2k + 1), h = s / 2, from the first terms of its own
+// expansion at k = 10.  What scales a whole patch is rounded once, scale and bias included: a
+// frame sums patches over many bins, where such errors add up and those of single bins average
+// out.
+__device__ __forceinline__ void series_terms(float s, float scale, float bias, float* term)
+{
+    constexpr float kInvFact[kTerms] = {1.0f, 5.0e-1f, 4.1666666666667e-2f, 1.3888888888889e-3f,
+                                        2.4801587301587e-5f, 2.7557319223986e-7f,
+                                        2.0876756987868e-9f, 1.1470745597729e-11f,
+                                        4.7794773323874e-14f, 1.5619206968586e-16f};   // 1 / (2k)!
+    const float h2 = 0.25f * s * s, g = 2.0f * h2, e = expf(-h2);
+    float A[kTerms];
+    float a = e * (1.0f / 21.0f) * (1.0f + g * (1.0f / 23.0f) * (1.0f + g * (1.0f / 25.0f)));
 #pragma unroll
-        for (int m = 0; m < 16; ++m) s_stirl[m] = c.stirl[m];    // constant indices: no local copy
+    for (int k = kTerms - 1; k >= 0; --k) {
+        a = fmaf(g, a, e) * (1.0f / (2 * k + 1));
+        A[k] = a;
     }
-    const int gl = threadIdx.x % G, grp = threadIdx.x / G;
+    const float r = 1.0f / A[0];
+    const float m = erff(0.5f * s), t0 = scale * m;
+    term[0] = t0 + fmaf(t0, bias, fmaf(scale, m, -t0));      // scale m (1 + bias), rounded once
+#pragma unroll
+    for (int k = 1; k < kTerms; ++k) term[k] = A[k] * (r * kInvFact[k]);
+}
+
+__device__ __forceinline__ bool series_axis(float off, float n, float frac, float s)
+{
+    const float c = fmaxf(fabsf((off + 0.5f) - frac), fabsf((off + (n - 0.5f)) - frac)) * s;
+    return c * s <= 4.47f && s <= 2.8f;   // sqrt(20); s far above for a point
+}
+
+// ex2.approx truncates: its mean relative error measured -2e-8 over (-1/4, 0), -3.2e-8 over
+// (-1, 0) and -5.0e-8 over (-7, 0).  Weighted by the masses, and with the rounding of log2 e, the
+// two factors of a bin took 7.7e-8 off the total of a patch (48,000 patches against 64 bits),
+// which the row factor puts back.
+constexpr float kEx2Bias = 7.7e-8f;
+
+template <int MODE>
+__device__ __forceinline__ void make_patch(const RasterConsts& c, const Decision& r, PatchDepo& out)
+{
+    PatchDepo p;
+    if (!r.ok || !(r.qatt > 0.0f)) {                      // nothing, or Q' underflowed
+        out.nr = 0;
+        return;
+    }
+    p.r_lo = r.r_lo;
+    p.nr = r.r_hi - r.r_lo + 1;
+    p.k_lo = r.k_lo;
+    p.nt = r.k_hi - r.k_lo + 1;
+    p.off_p = offset_float((int64_t)r.r_lo - r.i0p);
+    p.off_t = offset_float((int64_t)r.k_lo - r.i0t);
+    edge_axis(r.sp, c.dp_f, r.frac_p, p.frac_p, p.s_p);
+    edge_axis(r.st, c.dt_f, r.frac_t, p.frac_t, p.s_t);
+    p.qw = r.qw;
+    p.qatt = r.qatt;
+    p.inv_q = 1.0f / r.qatt;
+    p.id = r.id;
+    // the exact binomial keeps the erfc form: its integer draws then stay as they are
+    p.series = MODE != 2 && series_axis(p.off_p, (float)p.nr, p.frac_p, p.s_p) &&
+               series_axis(p.off_t, (float)p.nt, p.frac_t, p.s_t);
+    if (MODE != 2 && p.series) {
+        series_terms(p.s_t, 1.0f, 0.0f, p.term[0]);
+        series_terms(p.s_p, p.qw, kEx2Bias, p.term[1]);
+    }
+    out = p;
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Shared memory of one warp: its depos, then per group of lanes the weights of a patch tile.  A
+// row record is the row's weight (MODE 1: with the row's words of the
+// Philox second round), a quad record the weights of the four ticks 4 (q_lo + i) .. (zero outside
+// the window; MODE 1: with the quad's Philox words), read with 16-byte loads.
+constexpr int kMaxQuads = (kWmax + 3 + 3) / 4;
+
+template <int MODE>
+struct TileLayout {
+    static constexpr int kRow = MODE == 1 ? 4 : 1;       // floats per row record
+    static constexpr int kQuad = MODE == 1 ? 8 : 4;      // floats per quad record
+    static constexpr int kGroupBytes = kMaxQuads * kQuad * 4 + kWmax * kRow * 4;
+};
+
+__host__ __device__ constexpr int raster_warp_smem(int mode, int depos_per_warp, int lanes_per_depo)
+{
+    return depos_per_warp * (int)sizeof(PatchDepo) +
+           (32 / lanes_per_depo) * (mode == 1 ? TileLayout<1>::kGroupBytes : TileLayout<0>::kGroupBytes);
+}
+
+// The depos [base, base + dpw) of one event, dpw <= 32, by one warp: each lane decides one, then
+// each group of G lanes rasterizes one depo at a time.  MODE is the fluctuation mode (0 mean, 1
+// normal approximation, 2 exact binomial).
+template <int G, int MODE>
+__device__ __forceinline__ void rasterize_warp(const RasterConsts& c, const DepoArrays& d,
+                                               float* __restrict__ grid, int* flags, int64_t base,
+                                               int dpw, unsigned char* smem, const float* stirl)
+{
+    static_assert(G == 8 || G == 16 || G == 32, "lanes per depo");
+    using L = TileLayout<MODE>;
+    constexpr int NG = 32 / G;
+    const int lane = threadIdx.x & 31, gl = lane % G, grp = lane / G;
     // the lanes of this group within its warp
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-    const int64_t base = blk * KD;
-    if (threadIdx.x < KD) {
+    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << (G & 31)) - 1u) << (lane & ~(G - 1)));
+    PatchDepo* dep = reinterpret_cast<PatchDepo*>(smem);
+    if (lane < dpw) {
+        const int64_t i = base + lane;
         Decision r;
         r.ok = 0;
-        const int64_t i = base + threadIdx.x;
         if (i < d.n) {
             r = decide(c, d, i, flags, true);
-            r.id = d.id[i];
+            if (r.ok) r.id = d.id[i];
         }
-        s_dec[threadIdx.x] = r;
+        make_patch<MODE>(c, r, dep[lane]);
     }
-    __syncthreads();
+    __syncwarp();
     // 16-byte reductions need 4-tick groups to start on 16-byte boundaries
     const bool vec4 = ((c.n_ticks & 3) == 0) && ((reinterpret_cast<uintptr_t>(grid) & 15) == 0);
-    float* wp = s_wp[grp];
-    float* wt = s_wt[grp];
-    float* ed = s_edge[grp];
+    float* quad = reinterpret_cast<float*>(smem + dpw * sizeof(PatchDepo) + grp * L::kGroupBytes);
+    float* row = quad + kMaxQuads * L::kQuad;
 
-    for (int i = grp; i < KD; i += NG) {
-        const Decision dd = s_dec[i];
-        if (!dd.ok || !(dd.qatt > 0.0f)) continue;    // nothing, or Q' underflowed
-        // u = offset_in_bins * bin / (sqrt(2) sigma); sigma == 0 puts all weight in the
-        // single bin of the window.
-        const float s_p = (dd.sp > 0.0f) ? c.dp_f / (1.41421356237309505f * dd.sp) : 0.0f;
-        const float s_t = (dd.st > 0.0f) ? c.dt_f / (1.41421356237309505f * dd.st) : 0.0f;
-        const float inv_q = 1.0f / dd.qatt;
+#pragma unroll 1
+    for (int i = grp; i < dpw; i += NG) {
+        const PatchDepo& pd = dep[i];
+        const int nr_all = pd.nr, nt_all = pd.nt;
+        const float off_p = pd.off_p, frac_p = pd.frac_p, s_p = pd.s_p, qw = pd.qw;
+        const float off_t = pd.off_t, frac_t = pd.frac_t, s_t = pd.s_t, inv_q = pd.inv_q;
 
-        for (int32_t r0 = dd.r_lo; r0 <= dd.r_hi; r0 += kWmax) {
-            const int nr = min(kWmax, dd.r_hi - r0 + 1);
-            for (int32_t k0 = dd.k_lo; k0 <= dd.k_hi; k0 += kWmax) {
-                const int nt = min(kWmax, dd.k_hi - k0 + 1);
-                // one erfc per bin edge: nr + 1 row edges and nt + 1 tick edges
-                for (int e = gl; e < nr + nt + 2; e += G) {
-                    float v;
-                    if (e <= nr) v = edge_erfc((int64_t)(r0 + e) - dd.i0p, dd.frac_p, s_p);
-                    else v = edge_erfc((int64_t)(k0 + e - nr - 1) - dd.i0t, dd.frac_t, s_t);
-                    ed[e] = v;
+#pragma unroll 1
+        for (int32_t ra = 0; ra < nr_all; ra += kWmax) {
+            const int nr = min(kWmax, nr_all - ra), r0 = pd.r_lo + ra;
+#pragma unroll 1
+            for (int32_t ka = 0; ka < nt_all; ka += kWmax) {
+                const int nt = min(kWmax, nt_all - ka), k0 = pd.k_lo + ka;
+                const int q_lo = k0 >> 2, nq = ((k0 + nt - 1) >> 2) - q_lo + 1;
+                const int koff = k0 & 3;                   // slot of tick k0
+                for (int q = gl; q < nq; q += G) {
+                    *reinterpret_cast<float4*>(quad + L::kQuad * q) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if constexpr (MODE == 1)
+                        *reinterpret_cast<uint4*>(quad + L::kQuad * q + 4) =
+                            philox_quad(c.keys, c.plane_id, pd.id, (uint32_t)(q_lo + q));
                 }
-                const int q_lo = k0 >> 2, q_hi = (k0 + nt - 1) >> 2;
-                const int nq = q_hi - q_lo + 1;
-                const int koff = k0 - 4 * q_lo;            // slot of tick k0
                 __syncwarp(gmask);
-                for (int e = gl; e < nr + 4 * nq; e += G) {
-                    if (e < nr) {
-                        wp[e] = dd.qw * ((dd.sp > 0.0f)
-                                    ? bin_mass((int64_t)(r0 + e) - dd.i0p, dd.frac_p, s_p, ed[e], ed[e + 1])
-                                    : 1.0f);
+                // the weight w of tick ka + i (row < 0) or of row ra + row into its record
+                auto put = [&](int i, int row_i, float w) {
+                    if (row_i < 0) {
+                        const int p = i + koff;
+                        quad[L::kQuad == 4 ? p : (p >> 2) * L::kQuad + (p & 3)] = w;
+                    } else if constexpr (MODE == 1) {
+                        const uint64_t h = philox_row(c.keys, pd.id, (uint32_t)(r0 + row_i));
+                        *reinterpret_cast<float4*>(row + 4 * row_i) =
+                            make_float4(w, __uint_as_float((uint32_t)(h >> 32)),
+                                        __uint_as_float((uint32_t)h), 0.0f);
                     } else {
-                        const int k = e - nr - koff;
-                        float w = 0.0f;
-                        if (k >= 0 && k < nt)
-                            w = (dd.st > 0.0f) ? bin_mass((int64_t)(k0 + k) - dd.i0t, dd.frac_t, s_t,
-                                                          ed[nr + 1 + k], ed[nr + 2 + k])
-                                               : 1.0f;
-                        wt[e - nr] = w;
+                        row[row_i] = w;
+                    }
+                };
+                if (MODE != 2 && pd.series) {
+                    const float bt = off_t + ((float)ka + 0.5f), bp = off_p + ((float)(ra - nt) + 0.5f);
+                    for (int e = gl; e < nt + nr; e += G) {
+                        const bool tick = e < nt;
+                        const float4* tm = reinterpret_cast<const float4*>(pd.term[tick ? 0 : 1]);
+                        const float sc = tick ? s_t : s_p;
+                        const float cc = (((tick ? bt : bp) + (float)e) - (tick ? frac_t : frac_p)) * sc;
+                        const float cs = cc * sc, y = cs * cs;
+                        const float4 t0 = tm[0], t1 = tm[1], t2 = tm[2];
+                        float p = fmaf(y, t2.y, t2.x);
+                        p = fmaf(y, p, t1.w);
+                        p = fmaf(y, p, t1.z);
+                        p = fmaf(y, p, t1.y);
+                        p = fmaf(y, p, t1.x);
+                        p = fmaf(y, p, t0.w);
+                        p = fmaf(y, p, t0.z);
+                        p = fmaf(y, p, t0.y);
+                        p = fmaf(y, p, 1.0f);
+                        put(e, tick ? -1 : e - nt,
+                            t0.x * (p * ex2_ftz(cc * (cc * -1.44269504088896341f))));
+                    }
+                } else {
+                    // One erfc per bin edge, signed by the side of the mean it lies on: the nt + 1
+                    // tick edges, then the nr + 1 row edges, each lane's next edge in the next
+                    // lane (G - 1 bins per round).  The mass of a bin from its signed edge terms
+                    // a, b (span_mass's three cases) is half their difference, plus 1 when the
+                    // mean lies between them.
+                    const float bt = off_t + (float)ka, bp = off_p + (float)(ra - (nt + 1));
+                    for (int e0 = 0; e0 <= nr + nt; e0 += G - 1) {
+                        const int e = e0 + gl;
+                        const bool tick = e <= nt;
+                        const float u = (((tick ? bt : bp) + (float)e) - (tick ? frac_t : frac_p)) *
+                                        (tick ? s_t : s_p);
+                        const float a = copysignf(erfcf(fabsf(u)), u);
+                        const float b = __shfl_down_sync(gmask, a, 1, G);
+                        if (gl == G - 1 || e == nt || e > nr + nt) continue;
+                        float w = 0.5f * (a - b);
+                        if (__float_as_int(a) < 0 && __float_as_int(b) >= 0) w += 1.0f;
+                        put(e, tick ? -1 : e - (nt + 1), tick ? w : w * qw);
                     }
                 }
                 __syncwarp(gmask);
-                if constexpr (BIN) {
+                if constexpr (MODE == 2) {
                     // one bin per lane: neighbouring ticks cost alike, so the group's lanes
                     // walk their CDFs side by side, and no lane chains four draws
                     const float inv_nt = 1.0f / (float)nt;
@@ -156,45 +312,47 @@ __device__ __forceinline__ void rasterize_block(const RasterConsts& c, const Dep
                         const int ir = (int)(((float)b + 0.5f) * inv_nt);
                         const int ik = b - ir * nt;
                         const int64_t r = r0 + ir;
-                        const float v = wp[ir] * wt[ik + koff];
+                        const float v = row[ir] * quad[ik + koff];
                         if (!(v > 0.0f)) continue;
                         atomicAdd(grid + r * c.n_ticks + (k0 + ik),
-                                  binomial_bin(c, dd, k0 + ik, r, v, inv_q, s_stirl));
+                                  binomial_bin(c, pd.qatt, pd.id, k0 + ik, r, v, inv_q, stirl));
                     }
                     __syncwarp(gmask);
                     continue;
                 }
-                const float inv_nq = 1.0f / (float)nq;
-                for (int item = gl; item < nr * nq; item += G) {
-                    const int ir = (int)(((float)item + 0.5f) * inv_nq);
-                    const int iq = item - ir * nq;
-                    const int64_t r = r0 + ir;
-                    const int kq = (q_lo + iq) * 4;
-                    const float w = wp[ir];
-                    const float4 t4 = reinterpret_cast<const float4*>(wt)[iq];
-                    float v[4] = {w * t4.x, w * t4.y, w * t4.z, w * t4.w};
-                    if (c.fluctuate == 1) {
+                // (row, 4-tick group) items, G apart: the row and group of an item advance by
+                // G / nq and G mod nq (no division per item)
+                const float inv_nq = rcp_approx((float)nq);
+                const int step_r = (int)(((float)G + 0.5f) * inv_nq), step_q = G - step_r * nq;
+                int ir = (int)(((float)gl + 0.5f) * inv_nq), iq = gl - ir * nq;
+                float* tile = grid + (int64_t)r0 * c.n_ticks + 4 * q_lo;
+#pragma unroll 1
+                while (ir < nr) {
+                    const float4 t4 = *reinterpret_cast<const float4*>(quad + L::kQuad * iq);
+                    float v[4];
+                    if constexpr (MODE == 1) {
                         // normal approximation to Binomial(Q', mean / Q'); zero-mean bins
                         // (outside the window) stay zero
-                        float z[4];
-                        box_muller4(philox(make_uint4((uint32_t)(q_lo + iq), (uint32_t)r, dd.id,
-                                                      c.plane_id), c.key0, c.key1), z);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float var = v[e] * (1.0f - v[e] * inv_q);
-                            v[e] = fmaxf(0.0f, fmaf(sqrt_fast(var), z[e], v[e]));
-                        }
+                        const float4 rr = *reinterpret_cast<const float4*>(row + 4 * ir);
+                        const uint4 qq = *reinterpret_cast<const uint4*>(quad + 8 * iq + 4);
+                        v[0] = rr.x * t4.x; v[1] = rr.x * t4.y; v[2] = rr.x * t4.z; v[3] = rr.x * t4.w;
+                        fluctuate4(philox_rest(qq, __float_as_uint(rr.y), __float_as_uint(rr.z),
+                                               c.keys), inv_q, v);
+                    } else {
+                        const float w = row[ir];
+                        v[0] = w * t4.x; v[1] = w * t4.y; v[2] = w * t4.z; v[3] = w * t4.w;
                     }
-                    float* dst = grid + r * c.n_ticks + kq;
+                    float* dst = tile + (int64_t)ir * c.n_ticks + 4 * iq;
                     if (vec4) {
                         atomicAdd(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
                     } else {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int ik = kq + e - k0;
-                            if (ik >= 0 && ik < nt) atomicAdd(dst + e, v[e]);
-                        }
+                        for (int e = 0; e < 4; ++e)
+                            if ((unsigned)(4 * iq + e - koff) < (unsigned)nt) atomicAdd(dst + e, v[e]);
                     }
+                    ir += step_r;
+                    iq += step_q;
+                    if (iq >= nq) { iq -= nq; ++ir; }
                 }
                 __syncwarp(gmask);
             }
@@ -202,45 +360,71 @@ __device__ __forceinline__ void rasterize_block(const RasterConsts& c, const Dep
     }
 }
 
-template <int KD, int G, bool BIN>
-__global__ void __launch_bounds__(kWarps * 32)
-k_rasterize(RasterConsts c, DepoArrays d, float* __restrict__ grid, int* flags)
+// The binomial's small-count table in shared memory.
+template <int MODE>
+__device__ __forceinline__ void load_stirling(const RasterConsts& c, float* s_stirl)
 {
-    rasterize_block<KD, G, BIN>(c, d, grid, flags, blockIdx.x);
+    if constexpr (MODE == 2) {
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int m = 0; m < 16; ++m) s_stirl[m] = c.stirl[m];    // constant indices: no local copy
+        }
+        __syncthreads();
+    }
+}
+
+template <int G, int MODE>
+__global__ void __launch_bounds__(kRasterWarps * 32, MODE == 2 ? 8 : 10)
+k_rasterize(RasterConsts c, DepoArrays d, float* __restrict__ grid, int* flags, int dpw)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ float s_stirl[MODE == 2 ? 16 : 1];
+    load_stirling<MODE>(c, s_stirl);
+    const int warp = threadIdx.x >> 5;
+    rasterize_warp<G, MODE>(c, d, grid, flags, ((int64_t)blockIdx.x * kRasterWarps + warp) * dpw, dpw,
+                            smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
 }
 
 // Several events of one plane: CTA b belongs to the event whose block range holds b.
-template <int KD, int G, bool BIN>
-__global__ void __launch_bounds__(kWarps * 32)
-k_rasterize_batch(RasterConsts c, BatchEvents ev, int* flags)
+template <int G, int MODE>
+__global__ void __launch_bounds__(kRasterWarps * 32)
+k_rasterize_batch(RasterConsts c, BatchEvents ev, int* flags, int dpw)
 {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ float s_stirl[MODE == 2 ? 16 : 1];
+    load_stirling<MODE>(c, s_stirl);
+    const int warp = threadIdx.x >> 5;
     int e = 0;
     while (e + 1 < ev.n && ev.block_start[e + 1] <= (int)blockIdx.x) ++e;
-    c.key0 = ev.key0[e];
-    c.key1 = ev.key1[e];
-    rasterize_block<KD, G, BIN>(c, ev.d[e], ev.grid[e], flags,
-                                (int64_t)blockIdx.x - ev.block_start[e]);
+    c.keys.set(ev.key0[e], ev.key1[e]);
+    rasterize_warp<G, MODE>(c, ev.d[e], ev.grid[e], flags,
+                            (((int64_t)blockIdx.x - ev.block_start[e]) * kRasterWarps + warp) * dpw, dpw,
+                            smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
 }
 
-// Every event of a batch over a work queue: each CTA pops (event, depo block) items until the
-// queue is empty (events of different planes carry their own constants).
-template <int KD, int G, bool BIN>
-__global__ void __launch_bounds__(kWarps * 32)
-k_rasterize_queue(QueueEvents q, int* queue)
+// Every event of a batch over a work queue: each warp pops (event, piece of dpw depos) items
+// until the queue is empty (events of different planes carry their own constants).
+template <int G, int MODE>
+__global__ void __launch_bounds__(kRasterWarps * 32)
+k_rasterize_queue(QueueEvents q, int* queue, int dpw)
 {
-    __shared__ int s_item;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ float s_stirl[MODE == 2 ? 16 : 1];
+    load_stirling<MODE>(q.c[0], s_stirl);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int total = q.block_start[q.n];
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(queue, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();                   // every thread has the item before s_item is reused
+        int piece = 0;
+        if (lane == 0) piece = atomicAdd(queue, 1);
+        piece = __shfl_sync(0xffffffffu, piece, 0);
+        const int item = piece / kRasterWarps;
         if (item >= total) break;
         int e = 0;
         while (e + 1 < q.n && q.block_start[e + 1] <= item) ++e;
-        rasterize_block<KD, G, BIN>(q.c[e], q.d[e], q.grid[e], q.flags[e],
-                                    (int64_t)item - q.block_start[e]);
-        __syncthreads();                   // the block's shared tiles are reused by the next item
+        rasterize_warp<G, MODE>(q.c[e], q.d[e], q.grid[e], q.flags[e],
+                                (((int64_t)item - q.block_start[e]) * kRasterWarps + piece % kRasterWarps) * dpw,
+                                dpw, smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
+        __syncwarp();                      // the warp's tile is reused by the next item
     }
 }
 
@@ -510,76 +694,89 @@ __global__ void k_windows(RasterConsts c, DepoArrays d, int32_t* __restrict__ ou
 
 }  // namespace
 
+// Tiles that can be set by hand or tried by the autotuner: depos per 8 warps (per 256 threads),
+// lanes per depo.
 bool raster_tile_supported(int depos_per_block, int lanes_per_depo)
 {
-#define WCSIM_TILE_CASE(KD, G) if (depos_per_block == KD && lanes_per_depo == G) return true;
-    WCSIM_RASTER_TILES(WCSIM_TILE_CASE)
-#undef WCSIM_TILE_CASE
-    return false;
+    const int lo = lanes_per_depo == 8 ? 32 : 64;
+    if (lanes_per_depo != 8 && lanes_per_depo != 16 && lanes_per_depo != 32) return false;
+    return depos_per_block >= lo && depos_per_block <= 256 && (depos_per_block & (depos_per_block - 1)) == 0;
 }
+
+RasterTile raster_tile(const RasterConsts& c, int64_t n_depos)
+{
+    if (c.depos_per_block > 0) return {c.depos_per_block / 8, c.lanes_per_depo};
+    // One depo per warp for the exact binomial's long serial walks, two above 64k depos (2000
+    // depos: 76 us against 210 with 4 x 8 lanes; 30k: 427 / 472; 100k: 1288 with 2 x 16, 1330 with
+    // 1 x 32, 1326 with 4 x 8).  Else 8 lanes per depo, and more depos per warp (fewer, better
+    // filled decisions) as soon as there are warps enough for every SM (with fluctuation, 4 / 8 /
+    // 16 depos per warp: 2000 depos 10.9 / 15 / 21 us, 30k 25.2 / 25.3 / 29, 100k 58.5 / 56.0 /
+    // 58.0, 300k 148 / 132 / 128, 1M 466 / 404 / 378; 32 is slower throughout).
+    if (c.fluctuate == 2) return n_depos > 65536 ? RasterTile{2, 16} : RasterTile{1, 32};
+    return {n_depos > 196608 ? 16 : n_depos > 40000 ? 8 : 4, 8};
+}
+
+int rasterize_blocks(int64_t n_depos, int depos_per_warp)
+{
+    const int kd = kRasterWarps * depos_per_warp;
+    return (int)((n_depos + kd - 1) / kd);
+}
+
+// One launch of the instance for `lanes` and the fluctuation mode.
+#define WCSIM_RASTER_DISPATCH(KERNEL, lanes, mode, ...)                                        \
+    do {                                                                                       \
+        if (lanes == 8) {                                                                      \
+            if (mode == 2) { auto k = KERNEL<8, 2>; __VA_ARGS__; }                             \
+            else if (mode == 1) { auto k = KERNEL<8, 1>; __VA_ARGS__; }                        \
+            else { auto k = KERNEL<8, 0>; __VA_ARGS__; }                                       \
+        } else if (lanes == 16) {                                                              \
+            if (mode == 2) { auto k = KERNEL<16, 2>; __VA_ARGS__; }                            \
+            else if (mode == 1) { auto k = KERNEL<16, 1>; __VA_ARGS__; }                       \
+            else { auto k = KERNEL<16, 0>; __VA_ARGS__; }                                      \
+        } else {                                                                               \
+            if (mode == 2) { auto k = KERNEL<32, 2>; __VA_ARGS__; }                            \
+            else if (mode == 1) { auto k = KERNEL<32, 1>; __VA_ARGS__; }                       \
+            else { auto k = KERNEL<32, 0>; __VA_ARGS__; }                                      \
+        }                                                                                      \
+    } while (0)
 
 cudaError_t launch_rasterize(const RasterConsts& c, const DepoArrays& d, float* grid,
                              int* flags, cudaStream_t s)
 {
     if (d.n <= 0) return cudaSuccess;
-    if (!raster_tile_supported(c.depos_per_block, c.lanes_per_depo)) return cudaErrorInvalidValue;
-    const unsigned blocks = (unsigned)rasterize_blocks(d.n, c.depos_per_block);
-#define WCSIM_TILE_CASE(KD, G)                                                                 \
-    if (c.depos_per_block == KD && c.lanes_per_depo == G) {                                    \
-        if (c.fluctuate == 2)                                                                  \
-            k_rasterize<KD, G, true><<<blocks, kWarps * 32, 0, s>>>(c, d, grid, flags);        \
-        else                                                                                   \
-            k_rasterize<KD, G, false><<<blocks, kWarps * 32, 0, s>>>(c, d, grid, flags);       \
-    }
-    WCSIM_RASTER_TILES(WCSIM_TILE_CASE)
-#undef WCSIM_TILE_CASE
+    const RasterTile t = raster_tile(c, d.n);
+    const unsigned blocks = (unsigned)rasterize_blocks(d.n, t.depos_per_warp);
+    const int smem = kRasterWarps * raster_warp_smem(c.fluctuate, t.depos_per_warp, t.lanes_per_depo);
+    WCSIM_RASTER_DISPATCH(k_rasterize, t.lanes_per_depo, c.fluctuate,
+        k<<<blocks, kRasterWarps * 32, smem, s>>>(c, d, grid, flags, t.depos_per_warp));
     return cudaGetLastError();
 }
 
-int rasterize_blocks(int64_t n_depos, int depos_per_block)
-{
-    const int kd = depos_per_block > 0 ? depos_per_block : 64;
-    return (int)((n_depos + kd - 1) / kd);
-}
-
-cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev, int* flags,
-                                   cudaStream_t s)
+cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
+                                   const RasterTile& t, int* flags, cudaStream_t s)
 {
     const int blocks = ev.block_start[ev.n];
     if (blocks <= 0) return cudaSuccess;
-    if (!raster_tile_supported(c.depos_per_block, c.lanes_per_depo)) return cudaErrorInvalidValue;
-#define WCSIM_TILE_CASE(KD, G)                                                                 \
-    if (c.depos_per_block == KD && c.lanes_per_depo == G) {                                    \
-        if (c.fluctuate == 2)                                                                  \
-            k_rasterize_batch<KD, G, true><<<blocks, kWarps * 32, 0, s>>>(c, ev, flags);       \
-        else                                                                                   \
-            k_rasterize_batch<KD, G, false><<<blocks, kWarps * 32, 0, s>>>(c, ev, flags);      \
-    }
-    WCSIM_RASTER_TILES(WCSIM_TILE_CASE)
-#undef WCSIM_TILE_CASE
+    const int smem = kRasterWarps * raster_warp_smem(c.fluctuate, t.depos_per_warp, t.lanes_per_depo);
+    WCSIM_RASTER_DISPATCH(k_rasterize_batch, t.lanes_per_depo, c.fluctuate,
+        k<<<blocks, kRasterWarps * 32, smem, s>>>(c, ev, flags, t.depos_per_warp));
     return cudaGetLastError();
 }
 
-cudaError_t launch_rasterize_queue(const QueueEvents& q, int* queue, cudaStream_t s)
+cudaError_t launch_rasterize_queue(const QueueEvents& q, const RasterTile& t, int* queue,
+                                   cudaStream_t s)
 {
     const int total = q.block_start[q.n];
     if (q.n <= 0 || total <= 0) return cudaSuccess;
-    const RasterConsts& c = q.c[0];
-    if (!raster_tile_supported(c.depos_per_block, c.lanes_per_depo)) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), s);
     if (e) return e;
-#define WCSIM_TILE_CASE(KD, G)                                                                 \
-    if (c.depos_per_block == KD && c.lanes_per_depo == G) {                                    \
-        auto k = (c.fluctuate == 2) ? k_rasterize_queue<KD, G, true>                           \
-                                    : k_rasterize_queue<KD, G, false>;                         \
-        int per_sm = 0;                                                                        \
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWarps * 32, 0)))   \
-            return e;                                                                          \
-        const int resident = (per_sm > 0 ? per_sm : 1) * sm_count();                           \
-        k<<<total < resident ? total : resident, kWarps * 32, 0, s>>>(q, queue);               \
-    }
-    WCSIM_RASTER_TILES(WCSIM_TILE_CASE)
-#undef WCSIM_TILE_CASE
+    const int mode = q.c[0].fluctuate;
+    const int smem = kRasterWarps * raster_warp_smem(mode, t.depos_per_warp, t.lanes_per_depo);
+    WCSIM_RASTER_DISPATCH(k_rasterize_queue, t.lanes_per_depo, mode,
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRasterWarps * 32, smem))) return e;
+        const int resident = (per_sm > 0 ? per_sm : 1) * sm_count();
+        k<<<total < resident ? total : resident, kRasterWarps * 32, smem, s>>>(q, queue, t.depos_per_warp));
     return cudaGetLastError();
 }
 

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/wcsim.h"
+#include "rng.cuh"
 
 struct CUtensorMap_st;     // the driver's tensor map (cuda.h), by pointer only here
 
@@ -24,10 +25,11 @@ struct RasterConsts {
     int32_t n_ticks;
     int32_t fluctuate;
     int32_t renorm;                         // 1: each axis' weights divided by their window sum
-    uint32_t key0, key1, plane_id;
+    PhiloxKeys keys;                        // fluctuation stream
+    uint32_t plane_id;
     double DL, DT, v, tau;                  // FP64 parameters for the global gradients
-    int32_t depos_per_block;                // rasterization tile: depos per CTA and lanes
-    int32_t lanes_per_depo;                 // per depo (raster_tile_supported)
+    int32_t depos_per_block;                // rasterization tile set by hand or tuned: depos per
+    int32_t lanes_per_depo;                 // 8 warps and lanes per depo; 0: by raster_tile
     float stirl[16];                        // Stirling's remainder log m! - [(m + 1/2) log m
                                             // - m + 1/2 log 2 pi], m = 0..15 (exact binomial)
 };
@@ -77,15 +79,23 @@ cudaError_t launch_rasterize(const RasterConsts& c, const DepoArrays& d, float* 
                              int* flags, cudaStream_t s);
 cudaError_t launch_windows(const RasterConsts& c, const DepoArrays& d, int32_t* out,
                            int* flags, cudaStream_t s);
-// Rasterize several events of one plane in one launch (c.key0/key1 ignored: per event).
-cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev, int* flags,
+// How a rasterization splits the depos: depos per warp (at most 32) and lanes per depo.
+struct RasterTile {
+    int depos_per_warp, lanes_per_depo;
+};
+// The plane's tile if one was set, else the rule by the number of depos and fluctuation mode.
+RasterTile raster_tile(const RasterConsts& c, int64_t n_depos);
+// Rasterize several events of one plane in one launch (c.keys ignored: per event).
+cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
+                                   const RasterTile& t, int* flags, cudaStream_t s);
+// CTAs that n_depos depos take.
+int rasterize_blocks(int64_t n_depos, int depos_per_warp);
+// Rasterize every event of q in one persistent launch: warps pop pieces of the events' blocks
+// from *queue (zeroed here on the stream first) until all q.block_start[q.n] are done.  All
+// events use the tile t and the fluctuation mode of q.c[0].
+cudaError_t launch_rasterize_queue(const QueueEvents& q, const RasterTile& t, int* queue,
                                    cudaStream_t s);
-int rasterize_blocks(int64_t n_depos, int depos_per_block);
-// Rasterize every event of q in one persistent launch: CTAs pop (event, block) items from
-// *queue (zeroed here on the stream first) until all q.block_start[q.n] are done.  All events
-// use the tile (depos_per_block, lanes_per_depo) and fluctuation mode of q.c[0].
-cudaError_t launch_rasterize_queue(const QueueEvents& q, int* queue, cudaStream_t s);
-// Whether the rasterizers have an instance for this tile (depos per CTA, lanes per depo).
+// Whether a tile may be set (depos per 8 warps, lanes per depo).
 bool raster_tile_supported(int depos_per_block, int lanes_per_depo);
 // Adjoint of drift + rasterization (mean path, windows fixed): dgrid -> per-depo and global
 // gradients (dglobal must be zeroed by the caller).
