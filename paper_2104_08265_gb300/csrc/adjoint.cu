@@ -164,27 +164,30 @@ k_wire_adjoint_b(ConvDims d, const float2* __restrict__ tw2, const float2* __res
     }
 }
 
-template <int FIX>
-__global__ void __launch_bounds__(256, FIX == kPlanRuntime ? 2 : 3)
-k_rows_c2r_grid(ConvDims d, FftPlan p, const float2* __restrict__ shat, float* __restrict__ grid)
+template <int V>
+__global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
+k_rows_c2r_grid(ConvDims d, FftPlan p, const float2* __restrict__ shat, float* __restrict__ grid,
+                bool pairs)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
-    const int N = p.n;
     float2* X = reinterpret_cast<float2*>(smraw);
-    float2* Y = X + padded_len(N);
     // CTA b: impact j = b / npw, wires 2 (b mod npw) and the next one.  Adjacent wires of one
     // impact read adjacent 32-byte chunks of the blocked spectra.
     const int npw = (d.n_w + 1) / 2;
     const int j = blockIdx.x / npw, w0 = 2 * (blockIdx.x % npw), w1 = w0 + 1;
     const bool has1 = w1 < d.n_w;
     const int64_t slab = (int64_t)d.nkb * d.n_w * kBlockCols;
-    stage_herm_pair(shat + j * slab, shat + j * slab, w0, has1 ? w1 : w0, has1, d.n_w, d.nh, N, X);
-    __syncthreads();
-    const float2* z = run_row_plan<true, FIX, 256>(p, X, Y);
+    if (pairs) {
+        run_row_inverse_pairs<V>(p, X, shat + j * slab, w0, has1, d.n_w);
+    } else {
+        stage_herm_pair(shat + j * slab, shat + j * slab, w0, has1 ? w1 : w0, has1, d.n_w, d.nh, p.n, X);
+        __syncthreads();
+        run_row_inverse<V>(p, X);
+    }
     float* o0 = grid + ((int64_t)w0 * d.n_imp + j) * d.n_t;
     float* o1 = grid + ((int64_t)w1 * d.n_imp + j) * d.n_t;
-    const bool vec = ((d.n_t & 3) == 0) && ((reinterpret_cast<uintptr_t>(grid) & 15) == 0);
-    store_real_pair(z, o0, o1, d.n_t, has1, vec);
+    const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(grid) & 7) == 0);
+    store_real_pair(X, o0, o1, d.n_t, has1, vec);
 }
 
 // dL/dR_j(kw, kt) = conj(S_j^(kw, kt)) G^(kw, kt) / n and its Hermitian mirror (-kw, -kt)
@@ -318,17 +321,19 @@ cudaError_t launch_rows_c2r_grid(const ConvDims& d, const FftPlan& pt, const flo
                                  float* grid, cudaStream_t s)
 {
     if (g_attr.pending()) {
-        cudaError_t e = cudaFuncSetAttribute(k_rows_c2r_grid<kPlanRuntime>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (!e) e = cudaFuncSetAttribute(k_rows_c2r_grid<kPlan6000>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaError_t e = cudaSuccess;
+        for (int v = 0; v < kRowVariants && !e; ++v)
+            e = cudaFuncSetAttribute(WCSIM_ROW_KERNEL(k_rows_c2r_grid, v),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e) return e;
         g_attr.mark();
     }
     const int64_t n_ctas = (int64_t)d.n_imp * ((d.n_w + 1) / 2);
-    const int fix = fixed_plan_of(pt);
-    auto k = fix == kPlan6000 ? k_rows_c2r_grid<kPlan6000> : k_rows_c2r_grid<kPlanRuntime>;
-    k<<<(unsigned)n_ctas, 256, row_plan_smem(fix, pt.n), s>>>(d, pt, shat, grid);
+    const int t = row_block(pt, n_ctas);
+    auto k = WCSIM_ROW_KERNEL(k_rows_c2r_grid, row_variant(pt, t));
+    // mirrored pairs (run_row_inverse_pairs) from a few waves up
+    const bool pairs = row_pairs(pt, 0) && n_ctas > 8 * sm_count();
+    k<<<(unsigned)n_ctas, t, row_plan_smem(pt), s>>>(d, pt, shat, grid, pairs);
     return cudaGetLastError();
 }
 

@@ -9,10 +9,10 @@
 // batch lives at buf[pad(i) * B + c], where pad() inserts one slot every 16 elements so
 // that the stride-R writes of early passes do not pile onto one shared-memory bank.
 //
-// Plans come in two forms: a runtime plan (FftPlan: any length that factors into radices
-// <= 25, passes ping-ponging between two buffers) and compile-time plans (pass_fixed /
-// pass_fixed_inplace, all strides and divisors constants; the in-place form holds each
-// thread's butterfly inputs in registers across a barrier and needs one buffer).
+// Plans come in two forms: a runtime plan (FftPlan: any length that factors into radices <= 25)
+// and a compile-time plan (all strides and divisors constants).  A batch of sequences ping-pongs
+// between two buffers (run_plan); a single sequence is transformed in place in one buffer
+// (run_plan_inplace, run_plan_fixed).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -398,25 +398,26 @@ __device__ __forceinline__ void stage_herm_pair(const float2* __restrict__ s0,
     }
 }
 
-// Write the two real rows of an inverse real-pair transform held in the padded buffer z
-// (row 0 in .x, row 1 in .y; o1 ignored when !has1), ticks t < n_t.  With vec (rows 16-byte
-// aligned, n_t a multiple of 4) a thread writes 4 ticks of each row with one 16-byte store.
+// Write the two real rows of an inverse real-pair transform held in z (16-byte aligned; row 0 in
+// .x, row 1 in .y; o1 ignored when !has1), ticks t < n_t.  With vec (rows 8-byte aligned, n_t
+// even) a thread takes 2 ticks: consecutive lanes read consecutive 16 bytes of shared memory, free
+// of bank conflicts, and write 8 bytes of each row (four ticks per thread, with 16-byte stores,
+// read 32 bytes apart: the inverse FFT of dL/dS took 144 us with it).
 __device__ __forceinline__ void store_real_pair(const float2* z, float* __restrict__ o0,
                                                 float* __restrict__ o1, int n_t, bool has1,
                                                 bool vec)
 {
     if (vec) {
-        float4* p0 = reinterpret_cast<float4*>(o0);
-        float4* p1 = reinterpret_cast<float4*>(o1);
-        for (int q = threadIdx.x; q < (n_t >> 2); q += blockDim.x) {
-            const int i = pad16(4 * q);            // 4q .. 4q + 3 share one 16-slot group
-            const float2 a = z[i], b = z[i + 1], c = z[i + 2], e = z[i + 3];
-            p0[q] = make_float4(a.x, b.x, c.x, e.x);
-            if (has1) p1[q] = make_float4(a.y, b.y, c.y, e.y);
+        float2* p0 = reinterpret_cast<float2*>(o0);
+        float2* p1 = reinterpret_cast<float2*>(o1);
+        for (int q = threadIdx.x; q < (n_t >> 1); q += blockDim.x) {
+            const float4 a = reinterpret_cast<const float4*>(z)[q];       // ticks 2q, 2q + 1
+            p0[q] = make_float2(a.x, a.z);
+            if (has1) p1[q] = make_float2(a.y, a.w);
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[pad16(t)];
+            const float2 v = z[t];
             o0[t] = v.x;
             if (has1) o1[t] = v.y;
         }
@@ -425,8 +426,8 @@ __device__ __forceinline__ void store_real_pair(const float2* z, float* __restri
 
 // store_real_pair for a residual: o = M - target (one FP32 subtraction of the value
 // store_real_pair would write) for rows 0 (.x, target t0) and 1 (.y, t1); returns this
-// thread's FP32 sum of the squared residuals it wrote.  vec: rows and targets 16-byte
-// aligned, n_t a multiple of 4.
+// thread's FP32 sum of the squared residuals it wrote.  vec: rows and targets 8-byte aligned,
+// n_t even.
 __device__ __forceinline__ float store_residual_pair(const float2* z, float* __restrict__ o0,
                                                     float* __restrict__ o1,
                                                     const float* __restrict__ t0,
@@ -435,43 +436,40 @@ __device__ __forceinline__ float store_residual_pair(const float2* z, float* __r
 {
     float ss = 0.0f;
     if (vec) {
-        // the targets' 16-byte loads in batches of kU per row, issued before their use
+        // the targets' 8-byte loads in batches of kU per row, issued before their use
         constexpr int kU = 6;
-        const int nq = n_t >> 2;
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int nq = n_t >> 1;
+        const float2 zero = make_float2(0.f, 0.f);
         for (int base = threadIdx.x; base < nq; base += kU * blockDim.x) {
-            float4 ta[kU], tb[kU];
+            float2 ta[kU], tb[kU];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int q = base + u * blockDim.x;
                 ta[u] = tb[u] = zero;
                 if (q < nq) {
-                    ta[u] = __ldg(reinterpret_cast<const float4*>(t0) + q);
-                    if (has1) tb[u] = __ldg(reinterpret_cast<const float4*>(t1) + q);
+                    ta[u] = __ldg(reinterpret_cast<const float2*>(t0) + q);
+                    if (has1) tb[u] = __ldg(reinterpret_cast<const float2*>(t1) + q);
                 }
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int q = base + u * blockDim.x;
                 if (q < nq) {
-                    const int i = pad16(4 * q);
-                    const float2 a = z[i], b = z[i + 1], c = z[i + 2], e = z[i + 3];
-                    const float4 r0 = make_float4(__fsub_rn(a.x, ta[u].x), __fsub_rn(b.x, ta[u].y),
-                                                  __fsub_rn(c.x, ta[u].z), __fsub_rn(e.x, ta[u].w));
-                    reinterpret_cast<float4*>(o0)[q] = r0;
-                    ss += r0.x * r0.x + r0.y * r0.y + r0.z * r0.z + r0.w * r0.w;
+                    const float4 a = reinterpret_cast<const float4*>(z)[q];
+                    const float2 r0 = make_float2(__fsub_rn(a.x, ta[u].x), __fsub_rn(a.z, ta[u].y));
+                    reinterpret_cast<float2*>(o0)[q] = r0;
+                    ss += r0.x * r0.x + r0.y * r0.y;
                     if (has1) {
-                        const float4 r1 = make_float4(__fsub_rn(a.y, tb[u].x), __fsub_rn(b.y, tb[u].y),
-                                                      __fsub_rn(c.y, tb[u].z), __fsub_rn(e.y, tb[u].w));
-                        reinterpret_cast<float4*>(o1)[q] = r1;
-                        ss += r1.x * r1.x + r1.y * r1.y + r1.z * r1.z + r1.w * r1.w;
+                        const float2 r1 = make_float2(__fsub_rn(a.y, tb[u].x), __fsub_rn(a.w, tb[u].y));
+                        reinterpret_cast<float2*>(o1)[q] = r1;
+                        ss += r1.x * r1.x + r1.y * r1.y;
                     }
                 }
             }
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[pad16(t)];
+            const float2 v = z[t];
             const float r0 = __fsub_rn(v.x, t0[t]);
             o0[t] = r0;
             ss += r0 * r0;
@@ -495,26 +493,25 @@ __device__ __forceinline__ uint16_t adc_code(float m, float g, float p, float to
 }
 
 // store_real_pair for ADC codes: row 0 (.x) to o0, row 1 (.y) to o1, uint16.  With vec (rows
-// 8-byte aligned, n_t a multiple of 4) a thread writes 4 codes per row with one 8-byte store.
+// 4-byte aligned, n_t even) a thread writes 2 codes per row with one 4-byte store.
 __device__ __forceinline__ void store_real_pair_adc(const float2* z, uint16_t* __restrict__ o0,
                                                     uint16_t* __restrict__ o1, int n_t, bool has1,
                                                     bool vec, float g, float p, float top)
 {
     if (vec) {
-        uint2* p0 = reinterpret_cast<uint2*>(o0);
-        uint2* p1 = reinterpret_cast<uint2*>(o1);
-        for (int q = threadIdx.x; q < (n_t >> 2); q += blockDim.x) {
-            const int i = pad16(4 * q);
-            const float2 a = z[i], b = z[i + 1], c = z[i + 2], e = z[i + 3];
-            auto pack = [&](float u, float v) {
-                return (uint32_t)adc_code(u, g, p, top) | ((uint32_t)adc_code(v, g, p, top) << 16);
-            };
-            p0[q] = make_uint2(pack(a.x, b.x), pack(c.x, e.x));
-            if (has1) p1[q] = make_uint2(pack(a.y, b.y), pack(c.y, e.y));
+        uint32_t* p0 = reinterpret_cast<uint32_t*>(o0);
+        uint32_t* p1 = reinterpret_cast<uint32_t*>(o1);
+        auto pack = [&](float u, float v) {
+            return (uint32_t)adc_code(u, g, p, top) | ((uint32_t)adc_code(v, g, p, top) << 16);
+        };
+        for (int q = threadIdx.x; q < (n_t >> 1); q += blockDim.x) {
+            const float4 a = reinterpret_cast<const float4*>(z)[q];
+            p0[q] = pack(a.x, a.z);
+            if (has1) p1[q] = pack(a.y, a.w);
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[pad16(t)];
+            const float2 v = z[t];
             o0[t] = adc_code(v.x, g, p, top);
             if (has1) o1[t] = adc_code(v.y, g, p, top);
         }
@@ -542,17 +539,47 @@ __device__ __forceinline__ float2* run_plan(const FftPlan& p, const FirstLd& fir
     return dst;
 }
 
-// ------------------------------------------------------------------ compile-time plans
-// Apply the twiddles w^(r k), r = 1 .. R - 1, of a Stockham pass with stride NS to v[1 ..],
-// t = the pass's table + k (entry (r - 1) NS = w^(r k)).  Radix 15 loads only the entries of
-// r = 1, 5 and 10 and forms the rest as products of them (w^(3k) = w^(5k) conj(w^(2k)) and so
-// on, each at most three roundings away from correctly rounded table values), so a butterfly
-// reads 3 table entries instead of 14; other radices read every entry.
-template <int R, int NS, bool INV>
-__device__ __forceinline__ void apply_twiddles(float2* v, const float2* __restrict__ t)
+// ------------------------------------------------------------------ in-place plans
+// A single sequence in one shared buffer: in each pass every thread first loads the inputs of all
+// its butterflies into registers, the block synchronises, and the outputs are written over the
+// same buffer (one buffer per sequence instead of two, for more CTAs per SM).  The layout between
+// two passes pads each group of ns R outputs of the first by one slot when the group is even, so
+// that the first pass's stride-R writes spread over the banks; the groups divide the next pass's
+// strides, so every address is base + r step, with one base per butterfly (a pad of one slot per
+// 16 elements takes three operations per element where 16 does not divide the strides: a
+// 6250-point transform of 8000 rows took 184 us with it).  The input and the result are unpadded.
+//
+// A pass of the runtime plan reads its length and stride at run time; a fixed one has them as
+// template parameters.
+struct RtPass {
+    static constexpr bool kFew = false;
+    int n, ns, T;
+    uint32_t magic;
+    const float2* tw;
+    bool last;
+    __device__ __forceinline__ int div_ns(int j) const
+    {
+        return ns == 1 ? j : (int)__umulhi((uint32_t)j, magic);
+    }
+};
+template <int N, int NS, int THREADS, bool LAST>
+struct FixedPass {
+    static constexpr int n = N, ns = NS, T = THREADS;
+    static constexpr bool last = LAST, kFew = true;
+    const float2* tw;
+    __device__ __forceinline__ int div_ns(int j) const { return j / NS; }
+};
+
+// Apply the twiddles w^(r k), r = 1 .. R - 1, of a pass to v[1 ..]; tw the pass's table (entry
+// (r - 1) ns + k = w^(r k)).  FEW, radix 15: only the entries of r = 1, 5 and 10 are read and the
+// rest formed as products of them (w^(3k) = w^(5k) conj(w^(2k)) and so on, each at most three
+// roundings away from correctly rounded table values), 3 table entries instead of 14.
+template <int R, bool INV, bool FEW>
+__device__ __forceinline__ void apply_twiddles(float2* v, const float2* __restrict__ tw, int ns,
+                                               uint32_t k)
 {
-    if constexpr (R == 15) {
-        const float2 a = __ldg(t), b = __ldg(t + 4 * NS), c = __ldg(t + 9 * NS);
+    if constexpr (R == 15 && FEW) {
+        const float2 a = __ldg(tw + k), b = __ldg(tw + 4 * ns + k), c = __ldg(tw + 9 * ns + k);
         const float2 na = make_float2(a.x, -a.y);                  // conj: w^(-k)
         const float2 a2 = cmul(a, a), na2 = make_float2(a2.x, -a2.y);
         const float2 a3 = cmul(b, na2), a4 = cmul(b, na);
@@ -565,152 +592,363 @@ __device__ __forceinline__ void apply_twiddles(float2* v, const float2* __restri
         for (int r = 1; r < R; ++r) v[r] = twiddle<INV>(v[r], w[r]);
     } else {
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = twiddle<INV>(v[r], __ldg(t + (r - 1) * NS));
+        for (int r = 1; r < R; ++r) v[r] = twiddle<INV>(v[r], __ldg(tw + (r - 1) * ns + k));
     }
 }
 
-// One Stockham pass (single sequence) whose length N, radix R and stride NS are template
-// parameters, so that every divisor, stride and padded offset is a constant.  Same
-// arithmetic and twiddle table layout as pass_r.
-template <int R, bool INV, int N, int NS, class Ld, class St>
-__device__ __forceinline__ void pass_fixed(const Ld& ld, const St& st, const float2* __restrict__ tw)
+// The twiddles w^(r k) to va and their conjugates to vb.  Radix 15 reads the entries of r = 1, 2,
+// 5, 10 and 14 and forms the others as products of two of them: both halves of a pair see one
+// error here, which no longer averages out between them, so it is kept at one product.
+template <int R>
+__device__ __forceinline__ void pair_twiddles(float2* va, float2* vb, const float2* __restrict__ tw,
+                                              int ns, uint32_t k)
 {
-    constexpr int NB = N / R;
-    for (int j = threadIdx.x; j < NB; j += blockDim.x) {
-        const int q = j / NS, k = j - q * NS;
-        float2 v[R];
-        if constexpr (IsShared<Ld>::value && NB % 16 == 0) {
-            const int p0 = pad16(j);
+    float2 w[R];
+    if constexpr (R == 15) {
+        const float2 a = __ldg(tw + k), a2 = __ldg(tw + ns + k), b = __ldg(tw + 4 * ns + k);
+        const float2 c = __ldg(tw + 9 * ns + k), e = __ldg(tw + 13 * ns + k);
+        const float2 na = make_float2(a.x, -a.y), na2 = make_float2(a2.x, -a2.y);
+        w[1] = a;            w[2] = a2;            w[3] = cmul(b, na2);  w[4] = cmul(b, na);
+        w[5] = b;            w[6] = cmul(b, a);    w[7] = cmul(b, a2);   w[8] = cmul(c, na2);
+        w[9] = cmul(c, na);  w[10] = c;            w[11] = cmul(c, a);   w[12] = cmul(c, a2);
+        w[13] = cmul(e, na); w[14] = e;
+    } else {
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = ld.at(0, p0 + r * (NB + NB / 16));
-        } else {
+        for (int r = 1; r < R; ++r) w[r] = __ldg(tw + (r - 1) * ns + k);
+    }
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = ld(0, j + r * NB);
-        }
-        if constexpr (NS > 1) {
-            if (k > 0) apply_twiddles<R, NS, INV>(v, tw + k);
-        }
-        dft<R, INV>(v);
-        const int o = q * NS * R + k;
-        if constexpr (NS % 16 == 0 || (R == 16 && NS == 1)) {
-            constexpr int PS = (NS == 1) ? 1 : NS + NS / 16;
-            const int p0 = pad16(o);
-#pragma unroll
-            for (int r = 0; r < R; ++r) st.at(0, p0 + r * PS, v[r]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) st(0, o + r * NS, v[r]);
-        }
+    for (int r = 1; r < R; ++r) {
+        va[r] = twiddle<false>(va[r], w[r]);
+        vb[r] = twiddle<true>(vb[r], w[r]);
     }
 }
 
-// The three passes of a plan with radices R0, R1, R2 (p's twiddle table): first -> X,
-// X -> Y, Y -> X.  Returns X; ends with a block barrier.
-template <bool INV, int R0, int R1, int R2, class FirstLd>
-__device__ __forceinline__ float2* run_plan_fixed(const FftPlan& p, const FirstLd& first,
-                                                  float2* X, float2* Y)
+// One in-place pass of radix R, at most NI butterflies per thread; the block has P.T threads.
+// Ends with a block barrier.
+template <int R, bool INV, int NI, class P>
+__device__ __forceinline__ void pass_inplace(float2* buf, const P& p)
 {
-    constexpr int N = R0 * R1 * R2;
-    pass_fixed<R0, INV, N, 1>(first, SmemSt<0>{X}, p.tw + p.tw_off[0]);
-    __syncthreads();
-    pass_fixed<R1, INV, N, R0>(SmemLd<0>{X}, SmemSt<0>{Y}, p.tw + p.tw_off[1]);
-    __syncthreads();
-    pass_fixed<R2, INV, N, R0 * R1>(SmemLd<0>{Y}, SmemSt<0>{X}, p.tw + p.tw_off[2]);
-    __syncthreads();
-    return X;
-}
-
-// In-place variant of pass_fixed for a block of exactly T threads: every thread first loads
-// the inputs of all its butterflies (at most ceil(N / R / T)) into registers, the block
-// synchronises, and the outputs are written over the same buffer.  One buffer per sequence
-// instead of two, for more CTAs per SM.  Ends with a block barrier.
-template <int R, bool INV, int N, int NS, int T, class Ld>
-__device__ __forceinline__ void pass_fixed_inplace(const Ld& ld, float2* buf,
-                                                   const float2* __restrict__ tw)
-{
-    constexpr int NB = N / R;
-    constexpr int NI = (NB + T - 1) / T;
+    const int nb = p.n / R, ns = p.ns;
+    const int pad_in = (ns > 1 && (ns & 1) == 0) ? 1 : 0;
+    const int pad_out = (!p.last && ((ns * R) & 1) == 0) ? 1 : 0;
+    const int rd_step = nb + pad_in * p.div_ns(nb);
     float2 v[NI][R];
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
-        const int j = threadIdx.x + i * T;
-        if (j < NB) {
-            if constexpr (IsShared<Ld>::value && NB % 16 == 0) {
-                const int p0 = pad16(j);
+        const int j = threadIdx.x + i * p.T;
+        if (j < nb) {
+            const float2* src = buf + j + pad_in * p.div_ns(j);
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[i][r] = ld.at(0, p0 + r * (NB + NB / 16));
-            } else {
+            for (int r = 0; r < R; ++r) v[i][r] = src[r * rd_step];
+        } else {
+            // (unset, the values would be carried from one pass of the plan's loop to the next,
+            // and those of every radix stay live)
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[i][r] = ld(0, j + r * NB);
-            }
+            for (int r = 0; r < R; ++r) v[i][r] = make_float2(0.f, 0.f);
         }
     }
     __syncthreads();
-    const SmemSt<0> st{buf};
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
-        const int j = threadIdx.x + i * T;
-        if (j < NB) {
-            const int q = j / NS, k = j - q * NS;
-            if constexpr (NS > 1) {
-                if (k > 0) apply_twiddles<R, NS, INV>(v[i], tw + k);
-            }
+        const int j = threadIdx.x + i * p.T;
+        if (j < nb) {
+            const int q = p.div_ns(j), k = j - q * ns;
+            if (k > 0) apply_twiddles<R, INV, P::kFew>(v[i], p.tw, ns, (uint32_t)k);
             dft<R, INV>(v[i]);
-            const int o = q * NS * R + k;
-            if constexpr (NS % 16 == 0 || (R == 16 && NS == 1)) {
-                constexpr int PS = (NS == 1) ? 1 : NS + NS / 16;
-                const int p0 = pad16(o);
+            float2* dst = buf + q * (ns * R + pad_out) + k;
 #pragma unroll
-                for (int r = 0; r < R; ++r) st.at(0, p0 + r * PS, v[i][r]);
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) st(0, o + r * NS, v[i][r]);
-            }
+            for (int r = 0; r < R; ++r) dst[r * ns] = v[i][r];
         }
     }
     __syncthreads();
 }
 
-// The three passes of plan (R0, R1, R2) in place in X (padded layout on return), the first
-// reading through `first` (which may alias X, e.g. FlatLd over the staged input).  A block of
-// exactly T threads.  Returns X.
-template <bool INV, int R0, int R1, int R2, int T, class FirstLd>
-__device__ __forceinline__ float2* run_plan_fixed_inplace(const FftPlan& p, const FirstLd& first,
-                                                          float2* X)
+// The last pass of a forward transform of a real pair z = x0 + i x1, with the two half spectra
+// taken apart in registers: X0(k) = (Z(k) + conj Z(n - k)) / 2 to f[k] and X1(k) = (Z(k) - conj
+// Z(n - k)) / 2i to f[o1 + k], k <= n / 2.  With nb = n / R butterflies, outputs a + r nb of
+// butterfly a mirror those of butterfly nb - a, so a thread takes both (units a = 0 .. nb / 2, NI
+// per thread).  The twiddles of nb - a are those of a conjugated times W_R^r, and the factor W_R^r
+// turns its outputs by one: with v_b the transform without it, Z(n - a - r nb) = v_b[(R - r) mod R]
+// for every a, a = 0 (butterfly 0 twice) and a = nb / 2 included (whose values are written twice).
+// This saves writing the transform and reading it back, a fifth of the kernel's shared-memory
+// traffic.  f may overlap buf.  Ends without a barrier.
+template <int R, int NI, class P>
+__device__ __forceinline__ void last_pass_pairs(const float2* buf, const P& p, float2* f, int o1)
+{
+    const int nb = p.n / R, units = nb / 2 + 1;
+    const int pad_in = (p.ns > 1 && (p.ns & 1) == 0) ? 1 : 0;
+    const int rd_step = nb + pad_in;                   // ns == nb: one group
+    float2 va[NI][R], vb[NI][R];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int a = threadIdx.x + i * p.T;
+        if (a < units) {
+            const float2 *sa = buf + a, *sb = buf + (a ? nb - a : 0);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                va[i][r] = sa[r * rd_step];
+                vb[i][r] = sb[r * rd_step];
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) va[i][r] = vb[i][r] = make_float2(0.f, 0.f);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int a = threadIdx.x + i * p.T;
+        if (a < units) {
+            if (a > 0) pair_twiddles<R>(va[i], vb[i], p.tw, p.ns, (uint32_t)a);
+            dft<R, false>(va[i]);
+            dft<R, false>(vb[i]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 u = va[i][r], w = vb[i][(R - r) % R];
+                const float2 x0 = make_float2(0.5f * (u.x + w.x), 0.5f * (u.y - w.y));
+                const float2 x1 = make_float2(0.5f * (u.y + w.y), 0.5f * (w.x - u.x));
+                if (r <= (R - 1) / 2) {                // k = a + r nb <= n / 2
+                    f[a + r * nb] = x0;
+                    f[o1 + a + r * nb] = x1;
+                } else {                               // n - k, the conjugates
+                    f[(R - r) * nb - a] = make_float2(x0.x, -x0.y);
+                    f[o1 + (R - r) * nb - a] = make_float2(x1.x, -x1.y);
+                }
+            }
+        }
+    }
+}
+
+// The first pass of an inverse transform of a real pair, z(k) = X0(k) + i X1(k), from the two half
+// spectra: load(k, x0, x1) gives X0(k), X1(k), k <= n / 2, and z(n - k) = conj X0(k) + i conj
+// X1(k).  Inputs a + r nb of butterfly a mirror those of butterfly nb - a, so a thread that takes
+// both (units a = 0 .. nb / 2) reads each half-spectrum value once, all of them before the first
+// butterfly, and nothing is staged in shared memory.  Ends with a block barrier.
+template <int R, int NI, class P, class Load>
+__device__ __forceinline__ void first_pass_pairs(float2* buf, const P& p, const Load& load)
+{
+    const int nb = p.n / R, units = nb / 2 + 1;
+    const int pad = (!p.last && (R & 1) == 0) ? 1 : 0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int a = threadIdx.x + i * p.T;
+        if (a >= units) break;
+        float2 va[R], vb[R];
+#pragma unroll
+        for (int r = 0; r <= (R - 1) / 2; ++r) load(a + r * nb, va[r], vb[R - 1 - r]);
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) load((r + 1) * nb - a, vb[r], va[R - 1 - r]);
+        // (x0, x1) -> z(k) and z(n - k)
+        auto pair = [](float2& u, float2& w) {
+            const float2 x0 = u, x1 = w;
+            u = make_float2(x0.x - x1.y, x0.y + x1.x);
+            w = make_float2(x0.x + x1.y, x1.x - x0.y);
+        };
+#pragma unroll
+        for (int r = 0; r <= (R - 1) / 2; ++r) pair(va[r], vb[R - 1 - r]);
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) {
+            pair(vb[r], va[R - 1 - r]);
+            if (2 * (r + 1) == R && a == 0) va[R - 1 - r] = vb[r];     // k = n / 2 as it stands
+        }
+        dft<R, true>(va);
+        float2* dst = buf + a * (R + pad);
+#pragma unroll
+        for (int r = 0; r < R; ++r) dst[r] = va[r];
+        if (a > 0) {
+            dft<R, true>(vb);
+            dst = buf + (nb - a) * (R + pad);
+#pragma unroll
+            for (int r = 0; r < R; ++r) dst[r] = vb[r];
+        }
+    }
+    __syncthreads();
+}
+
+// Units of butterflies a and nb - a of radix R that a thread holds at once (32 complex values);
+// none above radix 16.
+__host__ __device__ constexpr int row_pair_units(int R) { return 16 / R; }
+
+// The passes of the compile-time plan (R0, R1, R2) for a block of exactly T threads, [FIRST, END)
+// of them.
+template <bool INV, int R0, int R1, int R2, int T, int FIRST = 0, int END = 3>
+__device__ __forceinline__ void run_plan_fixed(const FftPlan& p, float2* X)
 {
     constexpr int N = R0 * R1 * R2;
-    pass_fixed_inplace<R0, INV, N, 1, T>(first, X, p.tw + p.tw_off[0]);
-    pass_fixed_inplace<R1, INV, N, R0, T>(SmemLd<0>{X}, X, p.tw + p.tw_off[1]);
-    pass_fixed_inplace<R2, INV, N, R0 * R1, T>(SmemLd<0>{X}, X, p.tw + p.tw_off[2]);
-    return X;
+    constexpr int N0 = (N / R0 + T - 1) / T, N1 = (N / R1 + T - 1) / T, N2 = (N / R2 + T - 1) / T;
+    if constexpr (FIRST <= 0 && END > 0)
+        pass_inplace<R0, INV, N0>(X, FixedPass<N, 1, T, false>{p.tw + p.tw_off[0]});
+    if constexpr (FIRST <= 1 && END > 1)
+        pass_inplace<R1, INV, N1>(X, FixedPass<N, R0, T, false>{p.tw + p.tw_off[1]});
+    if constexpr (FIRST <= 2 && END > 2)
+        pass_inplace<R2, INV, N2>(X, FixedPass<N, R0 * R1, T, true>{p.tw + p.tw_off[2]});
 }
 
-// Plans with a compile-time variant: the 6000-point transform as radices 16, 25, 15.
-enum FixedPlan : int { kPlanRuntime = 0, kPlan6000 = 1 };
+// Butterflies of radix R that a thread of a runtime plan holds at once: at most 32 complex values
+// (64 registers).
+__host__ __device__ constexpr int row_butterflies(int R) { return R > 16 ? 1 : 32 / R; }
 
-__host__ inline int fixed_plan_of(const FftPlan& p)
+__device__ __forceinline__ RtPass rt_pass(const FftPlan& p, int i)
 {
-    if (p.n == 6000 && p.npass == 3 && p.radix[0] == 16 && p.radix[1] == 25 && p.radix[2] == 15)
-        return kPlan6000;
-    return kPlanRuntime;
+    return {p.n, p.ns[i], (int)blockDim.x, p.ns_magic[i], p.tw + p.tw_off[i], i + 1 == p.npass};
 }
 
-// All passes of a single-sequence plan for a block of T threads whose first pass reads the
-// staged input in Z (through FlatLd) and whose result may land in Z or W.  The compile-time
-// variant FIX (which must equal fixed_plan_of(p)) runs in place in Z alone; the runtime plan
-// ping-pongs between W and Z.  Returns the buffer holding the transform (padded layout).
-template <bool INV, int FIX, int T>
-__device__ __forceinline__ float2* run_row_plan(const FftPlan& p, float2* Z, float2* W)
+// Passes [first, end) of the runtime plan p, for a block of row_threads(p) threads.  (A plan of
+// one point has radix 1 and nothing to do.)
+template <bool INV>
+__device__ __forceinline__ void run_plan_inplace(const FftPlan& p, float2* X, int first, int end)
 {
-    if constexpr (FIX == kPlan6000) return run_plan_fixed_inplace<INV, 16, 25, 15, T>(p, FlatLd<0>{Z}, Z);
-    else return run_plan<INV, 0>(p, FlatLd<0>{Z}, W, Z);
+    for (int i = first; i < end; ++i) {
+        const RtPass a = rt_pass(p, i);
+        switch (p.radix[i]) {
+#define WCSIM_CASE(RR) case RR: pass_inplace<RR, INV, row_butterflies(RR)>(X, a); break;
+            WCSIM_FOR_EACH_RADIX(WCSIM_CASE)
+#undef WCSIM_CASE
+        }
+    }
 }
 
-// Shared bytes of a row kernel for transform length n: one padded buffer for the in-place
-// compile-time plans, two for the runtime plans.
-__host__ inline size_t row_plan_smem(int fix, int n)
+// Threads of a row kernel for plan p: every pass fits its butterflies, at least 128 (so that a
+// short transform still has the warps to hide its shared-memory latency), whole warps.
+__host__ inline int row_threads(const FftPlan& p)
 {
-    return (fix == kPlanRuntime ? 2 : 1) * (size_t)padded_len(n) * sizeof(float2);
+    int t = 128;
+    for (int i = 0; i < p.npass; ++i) {
+        const int nb = p.n / p.radix[i], ni = row_butterflies(p.radix[i]);
+        const int need = (nb + ni - 1) / ni;
+        if (need > t) t = need;
+    }
+    return (t + 31) & ~31;
 }
+
+// Row-kernel instances: the compile-time 6000-point plan (radices 16, 25, 15; 256 threads), and
+// the runtime plan for blocks of up to so many threads.  All keep one padded buffer per CTA and
+// 72 to 80 registers per thread (96 for the largest), so registers and shared memory give out
+// together: 24 warps per SM at 6000 points, 26 at 9600, where two ping-pong buffers of the same
+// plan left 8 to 16.
+enum RowVariant : int { kRow6000 = 0, kRow128, kRow256, kRow448, kRow704, kRowVariants };
+__host__ __device__ constexpr int row_max_threads(int v)
+{
+    return v == kRow128 ? 128 : v == kRow448 ? 448 : v == kRow704 ? 704 : 256;
+}
+__host__ __device__ constexpr int row_min_ctas(int v)
+{
+    return v == kRow128 ? 6 : v == kRow448 ? 2 : v == kRow704 ? 1 : 3;
+}
+
+__host__ inline bool is_plan6000(const FftPlan& p)
+{
+    return p.n == 6000 && p.npass == 3 && p.radix[0] == 16 && p.radix[1] == 25 && p.radix[2] == 15;
+}
+
+// Block of a row kernel for plan p over `ctas` CTAs: what the plan needs, at least 256 threads
+// when the CTAs are few for the SMs (a short transform's staging and stores are then what a CTA
+// waits for).
+__host__ inline int row_block(const FftPlan& p, int64_t ctas)
+{
+    if (is_plan6000(p)) return 256;
+    const int t = row_threads(p);
+    return t < 256 && ctas < 4 * (int64_t)sm_count() ? 256 : t;
+}
+
+__host__ inline RowVariant row_variant(const FftPlan& p, int block)
+{
+    if (is_plan6000(p)) return kRow6000;
+    return block <= 128 ? kRow128 : block <= 256 ? kRow256 : block <= 448 ? kRow448 : kRow704;
+}
+
+// Whether pass i of plan p, its first or last, can run on units of two mirrored butterflies: the
+// block that the other passes ask for holds them all.
+__host__ inline bool row_pairs(const FftPlan& p, int i)
+{
+    if (is_plan6000(p)) return true;
+    const int u = row_pair_units(p.radix[i]);
+    return p.radix[i] > 1 && u > 0 && p.n / p.radix[i] / 2 + 1 <= u * row_threads(p);
+}
+
+// Radices with units of two butterflies.
+#define WCSIM_FOR_EACH_PAIR_RADIX(X) \
+    X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(10) X(12) X(14) X(15) X(16)
+
+// Forward transform of the real pair staged in X.  pairs (row_pairs of the last pass): the two half
+// spectra in f and f + o1, which may overlap X, without a final barrier; else the transform in X.
+template <int V>
+__device__ __forceinline__ void run_row_forward(const FftPlan& p, float2* X, bool pairs, float2* f,
+                                                int o1)
+{
+    if constexpr (V == kRow6000) {
+        run_plan_fixed<false, 16, 25, 15, 256, 0, 2>(p, X);
+        if (pairs)
+            last_pass_pairs<15, 1>(X, FixedPass<6000, 400, 256, true>{p.tw + p.tw_off[2]}, f, o1);
+        else
+            run_plan_fixed<false, 16, 25, 15, 256, 2, 3>(p, X);
+    } else {
+        run_plan_inplace<false>(p, X, 0, pairs ? p.npass - 1 : p.npass);
+        if (pairs) {
+            const RtPass a = rt_pass(p, p.npass - 1);
+            switch (p.radix[p.npass - 1]) {
+#define WCSIM_CASE(RR) case RR: last_pass_pairs<RR, row_pair_units(RR)>(X, a, f, o1); break;
+                WCSIM_FOR_EACH_PAIR_RADIX(WCSIM_CASE)
+#undef WCSIM_CASE
+            }
+        }
+    }
+}
+
+// Inverse transform of the pair staged in X, in X.
+template <int V>
+__device__ __forceinline__ void run_row_inverse(const FftPlan& p, float2* X)
+{
+    if constexpr (V == kRow6000) run_plan_fixed<true, 16, 25, 15, 256>(p, X);
+    else run_plan_inplace<true>(p, X, 0, p.npass);
+}
+
+// Inverse transform of the real pair with half spectra at columns w0 and w0 + 1 (X1 = 0 when
+// !has1) of the blocked slab s into X, without staging them (row_pairs of the first pass).  It
+// loads with the few hundred threads that hold units: where the grid is many times the resident
+// CTAs that is faster (dL/dS of the 960 x 6000 plane 144 -> 126 us), where a launch is about one
+// wave the longer chain of a CTA shows (the frame's own inverse, 480 CTAs: 27 -> 37 us, so that
+// kernel stages).
+template <int V>
+__device__ __forceinline__ void run_row_inverse_pairs(const FftPlan& p, float2* X,
+                                                      const float2* __restrict__ s, int w0,
+                                                      bool has1, int n_w)
+{
+    const float2* col = s + (int64_t)w0 * kBlockCols;
+    auto load = [&](int k, float2& x0, float2& x1) {
+        const float2* q = col + (int64_t)(k >> 2) * n_w * kBlockCols + (k & 3);
+        x0 = __ldg(q);
+        x1 = has1 ? __ldg(q + kBlockCols) : make_float2(0.f, 0.f);
+    };
+    if constexpr (V == kRow6000) {
+        first_pass_pairs<16, 1>(X, FixedPass<6000, 1, 256, false>{p.tw}, load);
+        run_plan_fixed<true, 16, 25, 15, 256, 1, 3>(p, X);
+    } else {
+        const RtPass a = rt_pass(p, 0);
+        switch (p.radix[0]) {
+#define WCSIM_CASE(RR) case RR: first_pass_pairs<RR, row_pair_units(RR)>(X, a, load); break;
+            WCSIM_FOR_EACH_PAIR_RADIX(WCSIM_CASE)
+#undef WCSIM_CASE
+        }
+        run_plan_inplace<true>(p, X, 1, p.npass);
+    }
+}
+
+// Shared bytes of a row kernel for plan p: n complex values and one pad per even group of the
+// passes' layouts (at least padded_len(n), which the flat rows of the TMA stores are sized to).
+__host__ inline size_t row_plan_smem(const FftPlan& p)
+{
+    int len = padded_len(p.n);
+    for (int i = 0; i + 1 < p.npass; ++i) {
+        const int group = p.ns[i] * p.radix[i];
+        if ((group & 1) == 0 && p.n + p.n / group > len) len = p.n + p.n / group;
+    }
+    return (size_t)len * sizeof(float2);
+}
+
+// The instance of kernel template K for variant v.
+#define WCSIM_ROW_KERNEL(K, v)                                                                    \
+    ((v) == kRow6000 ? K<kRow6000> : (v) == kRow128 ? K<kRow128> : (v) == kRow256 ? K<kRow256>    \
+     : (v) == kRow448 ? K<kRow448> : K<kRow704>)
 
 }  // namespace wcsim

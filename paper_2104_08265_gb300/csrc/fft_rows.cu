@@ -6,8 +6,7 @@
 // rows_r2c (direct, the default) takes one pair of rows per CTA: both rows are loaded into
 // shared memory with batched 16-byte loads (scalar loads when rows are not 16-byte aligned),
 // a pair with no nonzero value stores zero spectra at once, and otherwise every pass of the
-// plan runs in shared memory (in place, in one buffer, for the compile-time 6000-point plan;
-// between two buffers for runtime plans); the CTA also asks L2 for the rows of the CTA
+// plan runs in place in one shared buffer; the CTA also asks L2 for the rows of the CTA
 // expected to follow it on the SM.  The two half spectra are separated into flat shared rows
 // and leave through TMA tensor box stores (per-thread stores with WCSIM_SPECTRA_TMA=0).
 // rows_r2c (staged, chosen by the autotuner or
@@ -29,7 +28,6 @@ namespace wcsim {
 namespace {
 
 constexpr int kStagedThreads = 512;
-constexpr int kDirectThreads = 256;
 constexpr size_t kMaxSmem = 227 * 1024;
 
 // First-pass source: element i of z = x0 + i x1 (zero beyond the frame), from a pair of rows
@@ -108,8 +106,9 @@ __device__ __forceinline__ bool stage_real_pair(float* g0, float* g1, int n_t, i
 // Separate the two real rows' half spectra and store them in the blocked layout (zeros in
 // the padding columns nh .. 4 nkb - 1).  Consecutive lanes take consecutive frequencies, so
 // the shared reads are free of conflicts and every 4 lanes fill one 32-byte sector per row.
-// The block size is a multiple of 16, so the output addresses and the padded shared indices
-// of k and N - k advance by constants from one iteration to the next.
+// The block size is a multiple of 16, so the output addresses and the shared indices of k and
+// N - k advance by constants from one iteration to the next.  PAD: z is padded (run_plan).
+template <bool PAD>
 __device__ __forceinline__ void store_pair_spectra(const ConvDims& d, const float2* z, int N,
                                                    int64_t r0, bool has1, float2* shat,
                                                    bool zero = false)
@@ -123,8 +122,8 @@ __device__ __forceinline__ void store_pair_spectra(const ConvDims& d, const floa
     const int64_t step = (int64_t)(blockDim.x / kBlockCols) * row;
     float2* q0 = shat + (int64_t)j0 * d.nkb * row + (k0 >> 2) * row + w0 * kBlockCols + (k0 & 3);
     float2* q1 = shat + (int64_t)j1 * d.nkb * row + (k0 >> 2) * row + w1 * kBlockCols + (k0 & 3);
-    const int dp = blockDim.x + (blockDim.x >> 4);                      // pad16 step
-    int pa = pad16(k0), pb = pad16(N - k0);
+    const int dp = blockDim.x + (PAD ? blockDim.x >> 4 : 0);
+    int pa = PAD ? pad16(k0) : k0, pb = PAD ? pad16(N - k0) : N - k0;
     for (int k = k0; k < nk; k += blockDim.x, q0 += step, q1 += step, pa += dp, pb -= dp) {
         float2 x0 = make_float2(0.f, 0.f), x1 = x0;
         if (k < nh && !zero) {
@@ -152,41 +151,32 @@ __device__ __forceinline__ float2* align128(float2* p)
 
 // Separate the pair's half spectra as store_pair_spectra does, into flat shared rows for the
 // TMA box stores: row 0's X0[k] at f[k], row 1's X1[k] at f[o1 + k], zeros for nh <= k < nk.
-// NI > 0: f may alias z; every thread first reads its NI frequencies k = tid + i T (NI T >= nh)
-// into registers, the block synchronises, then writes.  NI = 0: f and z are distinct buffers.
-// Ends with a proxy fence and a block barrier (the async proxy may then read f).
-template <int NI, int T>
+// f may alias z: every thread first reads its frequencies k = tid + i T, i < NI (NI T >= nh), into
+// registers, the block of T threads synchronises, then writes.  Ends with a proxy fence and a
+// block barrier (the async proxy may then read f).
+template <int NI>
 __device__ __forceinline__ void separate_flat(const float2* z, int N, int nh, int nk, int o1,
                                               float2* f)
 {
-    auto sep = [&](int k, float2& x0, float2& x1) {
-        const float2 a = z[pad16(k)];
-        const float2 b = z[k == 0 ? 0 : pad16(N - k)];
-        x0 = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-        x1 = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
-    };
-    if constexpr (NI > 0) {
-        float2 a0[NI], a1[NI];
+    const int T = blockDim.x;
+    float2 a0[NI], a1[NI];
 #pragma unroll
-        for (int i = 0; i < NI; ++i) {
-            const int k = threadIdx.x + i * T;
-            if (k < nh) sep(k, a0[i], a1[i]);
+    for (int i = 0; i < NI; ++i) {
+        const int k = threadIdx.x + i * T;
+        if (k < nh) {
+            const float2 a = z[k];
+            const float2 b = z[k == 0 ? 0 : N - k];
+            a0[i] = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
+            a1[i] = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
         }
-        __syncthreads();
+    }
+    __syncthreads();
 #pragma unroll
-        for (int i = 0; i < NI; ++i) {
-            const int k = threadIdx.x + i * T;
-            if (k < nh) {
-                f[k] = a0[i];
-                f[o1 + k] = a1[i];
-            }
-        }
-    } else {
-        for (int k = threadIdx.x; k < nh; k += T) {
-            float2 x0, x1;
-            sep(k, x0, x1);
-            f[k] = x0;
-            f[o1 + k] = x1;
+    for (int i = 0; i < NI; ++i) {
+        const int k = threadIdx.x + i * T;
+        if (k < nh) {
+            f[k] = a0[i];
+            f[o1 + k] = a1[i];
         }
     }
     for (int k = nh + threadIdx.x; k < nk; k += T) f[k] = f[o1 + k] = make_float2(0.f, 0.f);
@@ -262,7 +252,7 @@ k_rows_r2c_staged(ConvDims d, FftPlan p, const float* __restrict__ grid, float2*
             fence_proxy_async_smem();
             issue(i + 2);
         }
-        store_pair_spectra(d, z, N, r0, has1, shat);
+        store_pair_spectra<true>(d, z, N, r0, has1, shat);
         __syncthreads();
     }
     if (i < n_items && tid == 0) {
@@ -273,18 +263,17 @@ k_rows_r2c_staged(ConvDims d, FftPlan p, const float* __restrict__ grid, float2*
 
 // pf_ahead > 0: CTA b first asks L2 for the rows of pair b + pf_ahead (the CTA that will
 // most likely take over its slot once it retires), so that pair's first pass reads L2.
-// FIX: compile-time plan variant (fixed_plan_of(p)).
+// V: row_variant; pairs: row_pairs of the last pass.
 // bk > 0: the half spectra leave through TMA box stores of bk frequency blocks (map: the
 // blocked spectra, events along its last dimension); bk = 0: plain stores.
-template <int FIX>
-__global__ void __launch_bounds__(kDirectThreads, FIX == kPlanRuntime ? 2 : 3)
+template <int V>
+__global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
 k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __restrict__ shat,
-                  int pf_ahead, const __grid_constant__ CUtensorMap map, int bk)
+                  int pf_ahead, const __grid_constant__ CUtensorMap map, int bk, bool pairs)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
     const int N = p.n;
     float2* X = reinterpret_cast<float2*>(smraw);
-    float2* Y = X + padded_len(N);
     const int64_t n_rows = (int64_t)d.n_w * d.n_imp;
     const int64_t r0 = 2 * (int64_t)blockIdx.x;
     const bool has1 = r0 + 1 < n_rows;
@@ -303,53 +292,52 @@ k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __res
                                      d.clear_input != 0, X);
     // the transform of two all-zero rows is zero: store zero spectra and skip the passes
     if (!__syncthreads_or(any)) {
-        store_pair_spectra(d, X, N, r0, has1, shat, true);
+        store_pair_spectra<false>(d, X, N, r0, has1, shat, true);
         return;
     }
-    const float2* z = run_row_plan<false, FIX, kDirectThreads>(p, X, Y);
+    const int o1 = flat_row1(d.nkb), nk = kBlockCols * d.nkb;
+    float2* f = align128(X);
+    run_row_forward<V>(p, X, bk > 0 && pairs, f, o1);
     if (bk > 0) {
-        const int o1 = flat_row1(d.nkb);
-        if constexpr (FIX == kPlan6000) {
-            constexpr int NI = (6000 / 2 + 1 + kDirectThreads - 1) / kDirectThreads;
-            float2* f = align128(X);
-            separate_flat<NI, kDirectThreads>(z, N, d.nh, kBlockCols * d.nkb, o1, f);
-            if (threadIdx.x == 0) tma_store_pair(d, &map, f, o1, bk, r0, has1, blockIdx.y);
+        if (pairs) {
+            for (int k = d.nh + threadIdx.x; k < nk; k += blockDim.x) f[k] = f[o1 + k] = make_float2(0.f, 0.f);
+            fence_proxy_async_smem();
+            __syncthreads();
         } else {
-            float2* f = align128((z == X) ? Y : X);
-            separate_flat<0, kDirectThreads>(z, N, d.nh, kBlockCols * d.nkb, o1, f);
-            if (threadIdx.x == 0) tma_store_pair(d, &map, f, o1, bk, r0, has1, blockIdx.y);
+            // frequencies per thread: a runtime plan's block holds at least n / 32 threads
+            separate_flat<17>(X, N, d.nh, nk, o1, f);
         }
+        if (threadIdx.x == 0) tma_store_pair(d, &map, f, o1, bk, r0, has1, blockIdx.y);
         return;
     }
-    store_pair_spectra(d, z, N, r0, has1, shat);
+    store_pair_spectra<false>(d, X, N, r0, has1, shat);
 }
 
-template <int FIX>
-__global__ void __launch_bounds__(kDirectThreads, FIX == kPlanRuntime ? 2 : 3)
+template <int V>
+__global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
 k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
-    const int N = p.n;
     mt += blockIdx.y * d.ev_mt;              // event of a batched launch (0 otherwise)
     float* __restrict__ wave = waves.p[blockIdx.y];
     float2* X = reinterpret_cast<float2*>(smraw);
-    float2* Y = X + padded_len(N);
-    const int w0 = 2 * blockIdx.x, w1 = w0 + 1;
-    const bool has1 = w1 < d.n_w;
+    const int w0 = 2 * blockIdx.x;
+    const bool has1 = w0 + 1 < d.n_w;
     if (d.target && threadIdx.x == 0 && (d.n_t & 3) == 0 &&
         (reinterpret_cast<uintptr_t>(d.target) & 15) == 0) {
         // the target rows this CTA subtracts at the end: into L2 while it transforms
         bulk_prefetch_l2(d.target + (int64_t)w0 * d.n_t,
                          (uint32_t)((has1 ? 2 : 1) * d.n_t * sizeof(float)));
     }
-    stage_herm_pair(mt, mt, w0, has1 ? w1 : w0, has1, d.n_w, d.nh, N, X, d.noise_amp,
+    stage_herm_pair(mt, mt, w0, has1 ? w0 + 1 : w0, has1, d.n_w, d.nh, p.n, X, d.noise_amp,
                     d.noise_seed + (uint64_t)waves.ev[blockIdx.y], d.plane_id);
     __syncthreads();
-    const float2* z = run_row_plan<true, FIX, kDirectThreads>(p, X, Y);
+    run_row_inverse<V>(p, X);
+    const float2* z = X;
     if (d.adc_max > 0) {                       // digitized: uint16 codes at the same rows
         uint16_t* adc = reinterpret_cast<uint16_t*>(wave);
         uint16_t* a0 = adc + (int64_t)w0 * d.n_t;
-        const bool vec = ((d.n_t & 3) == 0) && ((reinterpret_cast<uintptr_t>(adc) & 7) == 0);
+        const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(adc) & 3) == 0);
         store_real_pair_adc(z, a0, a0 + d.n_t, d.n_t, has1, vec, d.adc_gain, d.adc_pedestal,
                             (float)d.adc_max);
         return;
@@ -357,8 +345,8 @@ k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
     float* o0 = wave + (int64_t)w0 * d.n_t;
     if (d.target) {                            // residual M - target, and 1/2 sum of squares
         const float* t0 = d.target + (int64_t)w0 * d.n_t;
-        const bool vec = ((d.n_t & 3) == 0) &&
-                         (((reinterpret_cast<uintptr_t>(wave) | reinterpret_cast<uintptr_t>(d.target)) & 15) == 0);
+        const bool vec = ((d.n_t & 1) == 0) &&
+                         (((reinterpret_cast<uintptr_t>(wave) | reinterpret_cast<uintptr_t>(d.target)) & 7) == 0);
         float ss = store_residual_pair(z, o0, o0 + d.n_t, t0, t0 + d.n_t, d.n_t, has1, vec);
         if (d.loss) {                          // one FP64 addition per warp (no static
 #pragma unroll                                         // shared memory: see attrs())
@@ -367,19 +355,19 @@ k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
         }
         return;
     }
-    const bool vec = ((d.n_t & 3) == 0) && ((reinterpret_cast<uintptr_t>(wave) & 15) == 0);
+    const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(wave) & 7) == 0);
     store_real_pair(z, o0, o0 + d.n_t, d.n_t, has1, vec);
 }
 
 // CTAs of the direct R2C kernel k resident on the whole GPU with smem bytes each, when its
 // rows may be prefetched with bulk copies (16-byte aligned rows); 0 otherwise.
 template <class K>
-int r2c_prefetch_ahead(const ConvDims& d, const float* grid, K k, size_t smem)
+int r2c_prefetch_ahead(const ConvDims& d, const float* grid, K k, int threads, size_t smem)
 {
     if ((d.n_t % 4) != 0 || (reinterpret_cast<uintptr_t>(grid) & 15) != 0) return 0;
     if (d.ev_grid % 4 != 0) return 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kDirectThreads, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -390,7 +378,7 @@ int r2c_prefetch_ahead(const ConvDims& d, const float* grid, K k, size_t smem)
 // and its box size, or bk = 0 (plain stores) when disabled, unmappable, or when the flat rows
 // plus the clipped tail of the last box, from a 128-byte aligned start, do not fit one
 // padded_len(n) buffer.
-int r2c_store_map(const ConvDims& d, const FftPlan& pt, int fix, const float2* shat, int n_ev,
+int r2c_store_map(const ConvDims& d, const FftPlan& pt, const float2* shat, int n_ev,
                   CUtensorMap* map)
 {
     memset(map, 0, sizeof(*map));
@@ -398,7 +386,6 @@ int r2c_store_map(const ConvDims& d, const FftPlan& pt, int fix, const float2* s
     const int bk = blocked_box_kb(d.nkb);
     const int64_t span = (int64_t)((d.nkb + bk - 1) / bk) * bk * kBlockCols;
     if (kFlatSlack + flat_row1(d.nkb) + span > (int64_t)padded_len(pt.n)) return 0;
-    (void)fix;   // both plan variants write the flat rows into one padded_len(n) buffer
     if (!blocked_spectra_map(shat, d.n_w, d.nkb, d.n_imp, n_ev, d.ev_shat, map)) return 0;
     return bk;
 }
@@ -411,10 +398,12 @@ cudaError_t attrs()
     if (!g_attr.pending()) return cudaSuccess;
     const int mx = (int)kMaxSmem;
     cudaError_t e = cudaFuncSetAttribute(k_rows_r2c_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_direct<kPlanRuntime>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_direct<kPlan6000>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (!e) e = cudaFuncSetAttribute(k_rows_c2r<kPlanRuntime>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (!e) e = cudaFuncSetAttribute(k_rows_c2r<kPlan6000>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    for (int v = 0; v < kRowVariants && !e; ++v) {
+        e = cudaFuncSetAttribute(WCSIM_ROW_KERNEL(k_rows_r2c_direct, v),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        if (!e) e = cudaFuncSetAttribute(WCSIM_ROW_KERNEL(k_rows_c2r, v),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    }
     if (!e) g_attr.mark();
     return e;
 }
@@ -422,7 +411,7 @@ cudaError_t attrs()
 }  // namespace
 
 cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* grid,
-                            float2* shat, int* flags, cudaStream_t s)
+                            float2* shat, int* flags, cudaStream_t s, bool pairs)
 {
     cudaError_t e = attrs();
     if (e) return e;
@@ -435,13 +424,14 @@ cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* g
         k_rows_r2c_staged<<<grid_n, kStagedThreads, smem, s>>>(d, pt, grid, shat, flags);
     } else {
         // the kernel writes the grid only with d.clear_input (consume and clear)
-        const int fix = fixed_plan_of(pt);
-        auto k = fix == kPlan6000 ? k_rows_r2c_direct<kPlan6000> : k_rows_r2c_direct<kPlanRuntime>;
-        const size_t sm = row_plan_smem(fix, pt.n);
+        const int t = row_block(pt, n_pairs);
+        auto k = WCSIM_ROW_KERNEL(k_rows_r2c_direct, row_variant(pt, t));
+        const size_t sm = row_plan_smem(pt);
         CUtensorMap map;
-        const int bk = r2c_store_map(d, pt, fix, shat, 1, &map);
-        k<<<(unsigned)n_pairs, kDirectThreads, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
-                                                        r2c_prefetch_ahead(d, grid, k, sm), map, bk);
+        const int bk = r2c_store_map(d, pt, shat, 1, &map);
+        k<<<(unsigned)n_pairs, t, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
+                                           r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
+                                           pairs && row_pairs(pt, pt.npass - 1));
     }
     return cudaGetLastError();
 }
@@ -461,26 +451,28 @@ cudaError_t launch_rows_c2r_batch(const ConvDims& d, const FftPlan& pt, const fl
     cudaError_t e = attrs();
     if (e) return e;
     const dim3 grid((unsigned)((d.n_w + 1) / 2), (unsigned)n_ev);
-    const int fix = fixed_plan_of(pt);
-    auto k = fix == kPlan6000 ? k_rows_c2r<kPlan6000> : k_rows_c2r<kPlanRuntime>;
-    k<<<grid, kDirectThreads, row_plan_smem(fix, pt.n), s>>>(d, pt, mt, waves);
+    const int t = row_block(pt, (int64_t)grid.x * grid.y);
+    auto k = WCSIM_ROW_KERNEL(k_rows_c2r, row_variant(pt, t));
+    k<<<grid, t, row_plan_smem(pt), s>>>(d, pt, mt, waves);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rows_r2c_batch(const ConvDims& d, const FftPlan& pt, const float* grid,
                                   float2* shat, int n_ev, cudaStream_t s)
 {
+    constexpr bool pairs = true;
     cudaError_t e = attrs();
     if (e) return e;
     const int64_t n_pairs = ((int64_t)d.n_w * d.n_imp + 1) / 2;
     const dim3 g((unsigned)n_pairs, (unsigned)n_ev);
-    const int fix = fixed_plan_of(pt);
-    auto k = fix == kPlan6000 ? k_rows_r2c_direct<kPlan6000> : k_rows_r2c_direct<kPlanRuntime>;
-    const size_t sm = row_plan_smem(fix, pt.n);
+    const int t = row_block(pt, n_pairs * n_ev);
+    auto k = WCSIM_ROW_KERNEL(k_rows_r2c_direct, row_variant(pt, t));
+    const size_t sm = row_plan_smem(pt);
     CUtensorMap map;
-    const int bk = r2c_store_map(d, pt, fix, shat, n_ev, &map);
-    k<<<g, kDirectThreads, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
-                                    r2c_prefetch_ahead(d, grid, k, sm), map, bk);
+    const int bk = r2c_store_map(d, pt, shat, n_ev, &map);
+    k<<<g, t, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
+                       r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
+                                           pairs && row_pairs(pt, pt.npass - 1));
     return cudaGetLastError();
 }
 

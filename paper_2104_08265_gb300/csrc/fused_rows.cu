@@ -154,7 +154,9 @@ __device__ __forceinline__ float bin_mass_direct(int64_t koff, float frac, float
 
 // Store the half spectra of the two rows of wire w held in z (row 0 in .x, row 1 in .y after
 // the real-pair split) at impact positions s0 and s0 + 1 of the blocked layout
-// [n_imp][nkb][n_w][4] (zeros for the padding columns, or everywhere when `zero`).
+// [n_imp][nkb][n_w][4] (zeros for the padding columns, or everywhere when `zero`).  PAD: z is
+// padded (run_plan).
+template <bool PAD>
 __device__ __forceinline__ void store_wire_pair(const ConvDims& d, const float2* z, int N, int w,
                                                 int s0, bool has1, float2* shat, bool zero)
 {
@@ -165,8 +167,8 @@ __device__ __forceinline__ void store_wire_pair(const ConvDims& d, const float2*
     const int64_t step = (int64_t)(blockDim.x / kBlockCols) * row;
     float2* q0 = shat + (int64_t)s0 * slice + (k0 >> 2) * row + w * kBlockCols + (k0 & 3);
     float2* q1 = q0 + slice;
-    const int dp = blockDim.x + (blockDim.x >> 4);
-    int pa = pad16(k0), pb = pad16(N - k0);
+    const int dp = blockDim.x + (PAD ? blockDim.x >> 4 : 0);
+    int pa = PAD ? pad16(k0) : k0, pb = PAD ? pad16(N - k0) : N - k0;
     for (int k = k0; k < nk; k += blockDim.x, q0 += step, q1 += step, pa += dp, pb -= dp) {
         float2 x0 = make_float2(0.f, 0.f), x1 = x0;
         if (k < nh && !zero) {
@@ -181,9 +183,9 @@ __device__ __forceinline__ void store_wire_pair(const ConvDims& d, const float2*
 }
 
 // One CTA per (wire, pair of impact positions j, j + 1; the last of an odd count alone).
-// FIX: compile-time plan variant.
-template <int FIX>
-__global__ void __launch_bounds__(kFusedThreads, FIX == kPlanRuntime ? 2 : 3)
+// FIX: the compile-time 6000-point plan, in place; else the runtime plan, between two buffers.
+template <bool FIX>
+__global__ void __launch_bounds__(kFusedThreads, FIX ? 3 : 2)
 k_rows_r2c_fused(ConvDims d, FftPlan p, RasterConsts c, FusedBins b, float2* __restrict__ shat)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
@@ -330,11 +332,13 @@ k_rows_r2c_fused(ConvDims d, FftPlan p, RasterConsts c, FusedBins b, float2* __r
     }
     const int s0 = ja;
     if (!any) {                                        // nothing deposited: zero spectra
-        store_wire_pair(d, X, N, w, s0, has1, shat, true);
+        store_wire_pair<!FIX>(d, X, N, w, s0, has1, shat, true);
         return;
     }
-    const float2* z = run_row_plan<false, FIX, T>(p, X, Y);
-    store_wire_pair(d, z, N, w, s0, has1, shat, false);
+    const float2* z = X;
+    if constexpr (FIX) run_plan_fixed<false, 16, 25, 15, T>(p, X);
+    else z = run_plan<false, 0>(p, FlatLd<0>{X}, Y, X);
+    store_wire_pair<!FIX>(d, z, N, w, s0, has1, shat, false);
 }
 
 // Largest dynamic shared memory a launch of kernel k may ask for on the current device: the
@@ -356,26 +360,32 @@ cudaError_t attrs()
 {
     if (!g_attr.pending()) return cudaSuccess;
     int m0 = 0, m1 = 0;
-    cudaError_t e = max_dynamic_smem(k_rows_r2c_fused<kPlanRuntime>, &m0);
-    if (!e) e = max_dynamic_smem(k_rows_r2c_fused<kPlan6000>, &m1);
-    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_fused<kPlanRuntime>, cudaFuncAttributeMaxDynamicSharedMemorySize, m0);
-    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_fused<kPlan6000>, cudaFuncAttributeMaxDynamicSharedMemorySize, m1);
+    cudaError_t e = max_dynamic_smem(k_rows_r2c_fused<false>, &m0);
+    if (!e) e = max_dynamic_smem(k_rows_r2c_fused<true>, &m1);
+    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, m0);
+    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, m1);
     if (!e) g_attr.mark();
     return e;
+}
+
+// One buffer for the compile-time plan, two for the runtime plan.
+size_t fused_smem(const FftPlan& p)
+{
+    return is_plan6000(p) ? row_plan_smem(p) : 2 * (size_t)padded_len(p.n) * sizeof(float2);
 }
 
 }  // namespace
 
 bool fused_supported(const FftPlan& pt)
 {
-    const int fix = fixed_plan_of(pt);
+    const bool fix = is_plan6000(pt);
     int mx = 0;
-    if (max_dynamic_smem(fix == kPlan6000 ? k_rows_r2c_fused<kPlan6000>
-                                          : k_rows_r2c_fused<kPlanRuntime>, &mx) != cudaSuccess) {
+    if (max_dynamic_smem(fix ? k_rows_r2c_fused<true>
+                                          : k_rows_r2c_fused<false>, &mx) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return row_plan_smem(fix, pt.n) <= (size_t)mx;
+    return fused_smem(pt) <= (size_t)mx;
 }
 
 cudaError_t launch_bin_depos(const RasterConsts& c, const DepoArrays& d, int n_imp, int n_w,
@@ -403,9 +413,9 @@ cudaError_t launch_rows_r2c_fused(const ConvDims& d, const FftPlan& pt, const Ra
     b.cap = s.cap;
     const int npj = (d.n_imp + 1) / 2;
     const unsigned blocks = (unsigned)(d.n_w * npj);
-    const int fix = fixed_plan_of(pt);
-    auto k = fix == kPlan6000 ? k_rows_r2c_fused<kPlan6000> : k_rows_r2c_fused<kPlanRuntime>;
-    k<<<blocks, kFusedThreads, row_plan_smem(fix, pt.n), st>>>(d, pt, c, b, shat);
+    const bool fix = is_plan6000(pt);
+    auto k = fix ? k_rows_r2c_fused<true> : k_rows_r2c_fused<false>;
+    k<<<blocks, kFusedThreads, fused_smem(pt), st>>>(d, pt, c, b, shat);
     return cudaGetLastError();
 }
 
