@@ -879,7 +879,11 @@ wcsim_status wcsim_run_backward(wcsim_plane* pl, const wcsim_depos* depos, const
         e = cudaMemsetAsync(pl->grid, 0, (size_t)d.n_w * d.n_imp * d.n_t * sizeof(float), s);
         if (e) return cuda_fail(e, "grid reset");
     }
-    pl->grid_clean = false;             // the grid ends up holding dL/dS
+    // dL/dS goes into the grid, or, after a forward that kept the 2D spectra of S, over those (this
+    // backward is their last reader, and they hold more than a grid): the grid then stays the
+    // cleared one the forward left, and the next forward resets nothing (37 us for 960 x 6000)
+    float* dS = reuse && pl->s2d_valid && pl->s2d ? reinterpret_cast<float*>(pl->s2d) : pl->grid;
+    if (dS == pl->grid) pl->grid_clean = false;
     markb(pl, 1, s);
     if (!reuse) {
         RasterConsts c = make_consts(pl);
@@ -888,10 +892,10 @@ wcsim_status wcsim_run_backward(wcsim_plane* pl, const wcsim_depos* depos, const
             return cuda_fail(e, "rasterize launch");
     }
     markb(pl, 2, s);
-    if ((st = convolve_adjoint(pl, grad_wave, pl->grid, pl->grid, grad_resp_c64, stream, reuse,
+    if ((st = convolve_adjoint(pl, grad_wave, pl->grid, dS, grad_resp_c64, stream, reuse,
                                reuse && pl->s2d_valid)))
         return st;
-    return wcsim_rasterize_adjoint(pl, depos, pl->grid, grads, stream);
+    return wcsim_rasterize_adjoint(pl, depos, dS, grads, stream);
 }
 
 wcsim_status wcsim_plane_reserve_batch(wcsim_plane* pl, int32_t n_events)
