@@ -27,9 +27,7 @@
 namespace wcsim {
 namespace {
 
-constexpr int kRasterWarps = 4; // warps per block of the rasterizers
-constexpr int kWarps = 8;       // warps per block of the adjoint
-constexpr int kDepos = 64;      // depos per block of the adjoint
+constexpr int kRasterWarps = 4; // warps per block
 constexpr int kWmax = 32;       // weights per axis held per patch tile
 
 // Exact binomial fluctuation of the bin (row r, tick k) with mean v: x ~ Binomial(N, p) with
@@ -464,210 +462,215 @@ __device__ __forceinline__ void renorm_factors(const RasterConsts& c, const Deci
     }
 }
 
-// Per depo (a half warp each, so that the per-group tiles fit static shared memory):
-// recompute the patch weights and their mu / sigma derivatives, gather dL/dS over the patch
-// and apply the chain rule through Q' = Q exp(-t_d / tau), t_a = t + t_d and
-// sigma = sqrt(2 D t_d).  The global sums are reduced per block in FP64.
-template <bool RN>
-__global__ void __launch_bounds__(kWarps * 32, 3)
-k_depo_adjoint(RasterConsts c, DepoArrays d, const float* __restrict__ dgrid, DepoGrads g,
-               int* flags)
+// What the adjoint's lanes need of one depo (edges as in PatchDepo); after its patch, the terms of
+// the three global sums.
+struct __align__(16) AdjointDepo {
+    int32_t r_lo, nr, k_lo, nt;      // window; nr == 0: the depo adds nothing
+    float off_p, frac_p, s_p, isp;   // isp, ist: 1 / sigma, 0 for a point
+    float off_t, frac_t, s_t, ist;
+    float qatt, att, sp, st;         // Q', Q' / Q, the sigmas
+    float a_q, dsl, dst, pad;        // dL/dQ', dL/dsigma_L, dL/dsigma_T
+    float rn[8];                     // renorm_factors
+};
+constexpr int kAdjointQuad = 12;     // floats per quad record: weights, dw/dmu, dw/dsigma
+constexpr int kAdjointGroup = kMaxQuads * kAdjointQuad * 4 + kWmax * 16;   // bytes per group
+
+__host__ __device__ constexpr int adjoint_warp_smem(int depos_per_warp)
 {
-    // 8 lanes per depo (as the forward's default tile; 16 lanes took 84 against 74 us on the
-    // 960 x 6000 plane); patch tiles of at most kTile rows x kTile ticks
-    constexpr int G = 8, NG = kWarps * 32 / G, kTile = 32;
-    __shared__ Decision s_dec[kDepos];
-    // wp, dwp/dmu, dwp/dsig per row; wt, dwt/dmu, dwt/dsig per tick laid out on 4-tick
-    // groups (slot p is tick 4 q_lo + p, zero outside the window)
-    __shared__ float s_w[NG][3][kTile];
-    __shared__ __align__(16) float s_t[NG][3][kTile + 8];
-    // per bin edge u: erfc|u|, phi(u) = exp(-u^2) / sqrt(2 pi) and u phi(u); rows then ticks
-    __shared__ float s_e[NG][3][2 * (kTile + 1)];
-    // per depo, the FP32 factors of its terms in the three global sums (dL/dsigma_L,
-    // sigma_L; dL/dsigma_T, sigma_T; dL/dQ', Q'), zero for depos that add nothing
-    __shared__ float s_gt[kDepos][6];
-    // per depo, the renormalisation factors of its rows and ticks: 1 / T, dT/dmu, dT/dsigma
-    // (an instance of its own, so that the plain adjoint keeps its registers)
-    __shared__ float s_rn[RN ? kDepos : 1][6];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gl = threadIdx.x % G, grp = threadIdx.x / G;
+    return depos_per_warp * (int)sizeof(AdjointDepo) + 4 * kAdjointGroup;
+}
+
+// Adjoint of drift and rasterization, split as the rasterizer: a warp decides its own dpw depos,
+// then each group of 8 lanes takes one at a time: it recomputes the patch weights and their mu /
+// sigma derivatives (one erfc and one normal pdf per bin edge, each lane's next edge in the next
+// lane), gathers dL/dS over the patch and applies the chain rule through Q' = Q exp(-t_d / tau),
+// t_a = t + t_d and sigma = sqrt(2 D t_d).  The global sums are reduced per block in FP64.
+// Bound by instructions: a block whose first two warps decided for eight, kept the edge terms in
+// shared memory (58 KB per block, three blocks per SM) and divided for every item's row took 70 us
+// on 100k depos of the 960 x 6000 plane, this 56 us (2000 depos 12.5 / 8.8 us).  Depos per warp:
+// as the rasterizer, 16 above 64k depos, 8, 4 below 16k.  The order of every sum over a patch is
+// as it was: the per-depo results keep
+// their bits.
+template <bool RN>
+__global__ void __launch_bounds__(kRasterWarps * 32, 8)
+k_depo_adjoint(RasterConsts c, DepoArrays d, const float* __restrict__ dgrid, DepoGrads g,
+               int* flags, int dpw)
+{
+    constexpr int G = 8;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane % G, grp = lane / G;
     const unsigned gmask = ((1u << G) - 1u) << (lane & ~(G - 1));
-    const int64_t base = (int64_t)blockIdx.x * kDepos;
-    if (threadIdx.x < kDepos) {
-        Decision r;
-        r.ok = 0;
-        const int64_t i = base + threadIdx.x;
+    unsigned char* wsm = smraw + warp * adjoint_warp_smem(dpw);
+    AdjointDepo* dep = reinterpret_cast<AdjointDepo*>(wsm);
+    const int64_t base = ((int64_t)blockIdx.x * kRasterWarps + warp) * dpw;
+    if (lane < dpw) {
+        AdjointDepo p;
+        p.nr = 0;
+        p.nt = 0;
+        p.qatt = p.att = p.a_q = p.dsl = p.dst = p.sp = p.st = 0.0f;
+        const int64_t i = base + lane;
         if (i < d.n) {
-            r = decide(c, d, i, flags);
-            r.id = d.id[i];
+            const Decision r = decide(c, d, i, flags);
+            if (RN) renorm_factors(c, r, p.rn);
+            if (r.ok && r.qatt > 0.0f) {
+                p.r_lo = r.r_lo;
+                p.nr = r.r_hi - r.r_lo + 1;
+                p.k_lo = r.k_lo;
+                p.nt = r.k_hi - r.k_lo + 1;
+                p.off_p = offset_float((int64_t)r.r_lo - r.i0p);
+                p.off_t = offset_float((int64_t)r.k_lo - r.i0t);
+                edge_axis(r.sp, c.dp_f, r.frac_p, p.frac_p, p.s_p);
+                edge_axis(r.st, c.dt_f, r.frac_t, p.frac_t, p.s_t);
+                p.isp = (r.sp > 0.0f) ? 1.0f / r.sp : 0.0f;
+                p.ist = (r.st > 0.0f) ? 1.0f / r.st : 0.0f;
+                p.qatt = r.qatt;
+                p.att = r.qatt / d.q[i];
+                p.sp = r.sp;
+                p.st = r.st;
+            }
         }
-        s_dec[threadIdx.x] = r;
-        if (RN) renorm_factors(c, r, s_rn[threadIdx.x]);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) s_gt[threadIdx.x][k] = 0.0f;
+        dep[lane] = p;
     }
-    __syncthreads();
-    float* wp = s_w[grp][0];
-    float* wpm = s_w[grp][1];
-    float* wps = s_w[grp][2];
-    float* wt = s_t[grp][0];
-    float* wtm = s_t[grp][1];
-    float* wts = s_t[grp][2];
-    float* eE = s_e[grp][0];
-    float* eP = s_e[grp][1];
-    float* eU = s_e[grp][2];
+    __syncwarp();
+    float* quad = reinterpret_cast<float*>(wsm + dpw * sizeof(AdjointDepo) + grp * kAdjointGroup);
+    float* row = quad + kMaxQuads * kAdjointQuad;
     const bool vec4 = ((c.n_ticks & 3) == 0) && ((reinterpret_cast<uintptr_t>(dgrid) & 15) == 0);
 
-    for (int i = grp; i < kDepos; i += NG) {
+#pragma unroll 1
+    for (int i = grp; i < dpw; i += 32 / G) {
         const int64_t gi = base + i;
         if (gi >= d.n) break;
-        const Decision dd = s_dec[i];
+        AdjointDepo& pd = dep[i];
+        const int nr_all = pd.nr, nt_all = pd.nt;
+        const float off_p = pd.off_p, frac_p = pd.frac_p, s_p = pd.s_p, isp = pd.isp;
+        const float off_t = pd.off_t, frac_t = pd.frac_t, s_t = pd.s_t, ist = pd.ist;
         float a_q = 0.f, a_pm = 0.f, a_ps = 0.f, a_tm = 0.f, a_ts = 0.f;
-        if (dd.ok && dd.qatt > 0.0f) {
-            const float s_p = (dd.sp > 0.0f) ? c.dp_f / (1.41421356237309505f * dd.sp) : 0.0f;
-            const float s_t = (dd.st > 0.0f) ? c.dt_f / (1.41421356237309505f * dd.st) : 0.0f;
-            const float isp = (dd.sp > 0.0f) ? 1.0f / dd.sp : 0.0f;
-            const float ist = (dd.st > 0.0f) ? 1.0f / dd.st : 0.0f;
-            // renormalised weights w / T and their derivatives by the quotient rule,
-            // (dw - (w / T) dT) / T (the identity when renormalisation is off)
-            const float* rn = s_rn[RN ? i : 0];
-            for (int32_t r0 = dd.r_lo; r0 <= dd.r_hi; r0 += kTile) {
-                const int nr = min(kTile, dd.r_hi - r0 + 1);
-                for (int32_t k0 = dd.k_lo; k0 <= dd.k_hi; k0 += kTile) {
-                    const int nt = min(kTile, dd.k_hi - k0 + 1);
-                    const int q_lo = k0 >> 2, q_hi = (k0 + nt - 1) >> 2, nq = q_hi - q_lo + 1;
-                    const int koff = k0 - 4 * q_lo;        // slot of tick k0
-                    // edge terms: nr + 1 row edges, nt + 1 tick edges
-                    for (int e = gl; e < nr + nt + 2; e += G) {
-                        const float u = (e <= nr) ? ((float)((int64_t)(r0 + e) - dd.i0p) - dd.frac_p) * s_p
-                                                  : ((float)((int64_t)(k0 + e - nr - 1) - dd.i0t) - dd.frac_t) * s_t;
-                        const float ph = 0.398942280401432678f * expf(-u * u);
-                        eE[e] = erfcf(fabsf(u));
-                        eP[e] = ph;
-                        eU[e] = u * ph;
+#pragma unroll 1
+        for (int32_t ra = 0; ra < nr_all; ra += kWmax) {
+            const int nr = min(kWmax, nr_all - ra), r0 = pd.r_lo + ra;
+#pragma unroll 1
+            for (int32_t ka = 0; ka < nt_all; ka += kWmax) {
+                const int nt = min(kWmax, nt_all - ka), k0 = pd.k_lo + ka;
+                const int q_lo = k0 >> 2, nq = ((k0 + nt - 1) >> 2) - q_lo + 1;
+                const int koff = k0 & 3;               // slot of tick k0
+                for (int q = gl; q < 3 * nq; q += G)
+                    *reinterpret_cast<float4*>(quad + 4 * q) = make_float4(0.f, 0.f, 0.f, 0.f);
+                __syncwarp(gmask);
+                // w = Phi(b') - Phi(a'); dw/dmu = -(phi(b') - phi(a')) / sigma;
+                // dw/dsigma = -(b' phi(b') - a' phi(a')) / sigma, with b' = sqrt(2) ub.
+                // Renormalised weights w / T and their derivatives by the quotient rule,
+                // (dw - (w / T) dT) / T.
+                const float bt = off_t + (float)ka, bp = off_p + (float)(ra - (nt + 1));
+                for (int e0 = 0; e0 <= nr + nt; e0 += G - 1) {
+                    const int e = e0 + gl;
+                    const bool tick = e <= nt;
+                    const float u = (((tick ? bt : bp) + (float)e) - (tick ? frac_t : frac_p)) *
+                                    (tick ? s_t : s_p);
+                    const float ph = 0.398942280401432678f * expf(-u * u), up = u * ph;
+                    const float a = copysignf(erfcf(fabsf(u)), u);
+                    const float b = __shfl_down_sync(gmask, a, 1, G);
+                    const float phb = __shfl_down_sync(gmask, ph, 1, G);
+                    const float upb = __shfl_down_sync(gmask, up, 1, G);
+                    if (gl == G - 1 || e == nt || e > nr + nt) continue;
+                    float w = 0.5f * (a - b);
+                    if (__float_as_int(a) < 0 && __float_as_int(b) >= 0) w += 1.0f;
+                    const float is = tick ? ist : isp;
+                    const float m = -(phb - ph), sg = -1.41421356237309505f * (upb - up);
+                    float wn = w, wm = m * is, ws = sg * is;
+                    if (RN) {
+                        const float* rn = pd.rn + (tick ? 3 : 0);
+                        wn = w * rn[0];
+                        wm = (m * is - wn * rn[1]) * rn[0];
+                        ws = (sg * is - wn * rn[2]) * rn[0];
                     }
-                    __syncwarp(gmask);
-                    // w = Phi(b') - Phi(a'); dw/dmu = -(phi(b') - phi(a')) / sigma;
-                    // dw/dsigma = -(b' phi(b') - a' phi(a')) / sigma, with b' = sqrt(2) ub
-                    for (int e = gl; e < nr + 4 * nq; e += G) {
-                        if (e < nr) {
-                            float w = 1.0f, m = 0.0f, sg = 0.0f;
-                            if (dd.sp > 0.0f) {
-                                w = bin_mass((int64_t)(r0 + e) - dd.i0p, dd.frac_p, s_p, eE[e], eE[e + 1]);
-                                m = -(eP[e + 1] - eP[e]);
-                                sg = -1.41421356237309505f * (eU[e + 1] - eU[e]);
-                            }
-                            if (RN) {
-                                const float wn = w * rn[0];
-                                wp[e] = wn;
-                                wpm[e] = (m * isp - wn * rn[1]) * rn[0];
-                                wps[e] = (sg * isp - wn * rn[2]) * rn[0];
-                            } else {
-                                wp[e] = w;
-                                wpm[e] = m * isp;
-                                wps[e] = sg * isp;
-                            }
-                        } else {
-                            const int k = e - nr - koff, a = nr + 1 + k;
-                            float w = 0.0f, m = 0.0f, sg = 0.0f;
-                            if (k >= 0 && k < nt) {
-                                if (dd.st > 0.0f) {
-                                    w = bin_mass((int64_t)(k0 + k) - dd.i0t, dd.frac_t, s_t, eE[a], eE[a + 1]);
-                                    m = -(eP[a + 1] - eP[a]);
-                                    sg = -1.41421356237309505f * (eU[a + 1] - eU[a]);
-                                } else {
-                                    w = 1.0f;
-                                }
-                            }
-                            if (RN) {
-                                const float wn = w * rn[3];
-                                wt[e - nr] = wn;
-                                wtm[e - nr] = (m * ist - wn * rn[4]) * rn[3];
-                                wts[e - nr] = (sg * ist - wn * rn[5]) * rn[3];
-                            } else {
-                                wt[e - nr] = w;
-                                wtm[e - nr] = m * ist;
-                                wts[e - nr] = sg * ist;
-                            }
-                        }
-                    }
-                    __syncwarp(gmask);
-                    if (vec4) {
-                        // (row, 4-tick group) items: one 16-byte load of dL/dS per item
-                        const float inv_nq = 1.0f / (float)nq;
-                        for (int item = gl; item < nr * nq; item += G) {
-                            const int ir = (int)(((float)item + 0.5f) * inv_nq);
-                            const int iq = item - ir * nq;
-                            const int kq = (q_lo + iq) * 4;
-                            const float4 sv = __ldg(reinterpret_cast<const float4*>(
-                                dgrid + (int64_t)(r0 + ir) * c.n_ticks + kq));
-                            const float4 w4 = reinterpret_cast<const float4*>(wt)[iq];
-                            const float4 m4 = reinterpret_cast<const float4*>(wtm)[iq];
-                            const float4 g4 = reinterpret_cast<const float4*>(wts)[iq];
-                            const float A = sv.x * w4.x + sv.y * w4.y + sv.z * w4.z + sv.w * w4.w;
-                            const float B = sv.x * m4.x + sv.y * m4.y + sv.z * m4.z + sv.w * m4.w;
-                            const float C = sv.x * g4.x + sv.y * g4.y + sv.z * g4.z + sv.w * g4.w;
-                            const float pw = wp[ir];
-                            a_q += pw * A;
-                            a_pm += wpm[ir] * A;
-                            a_ps += wps[ir] * A;
-                            a_tm += pw * B;
-                            a_ts += pw * C;
-                        }
+                    if (tick) {
+                        const int p = e + koff;
+                        float* q = quad + (p >> 2) * kAdjointQuad + (p & 3);
+                        q[0] = wn;
+                        q[4] = wm;
+                        q[8] = ws;
                     } else {
-                        const float inv_nt = 1.0f / (float)nt;
-                        for (int b = gl; b < nr * nt; b += G) {
-                            const int ir = (int)(((float)b + 0.5f) * inv_nt);
-                            const int ik = b - ir * nt;
-                            const float sv = __ldg(dgrid + (int64_t)(r0 + ir) * c.n_ticks + (k0 + ik));
-                            const float pw = wp[ir], tw = wt[ik + koff];
-                            a_q += sv * pw * tw;
-                            a_pm += sv * wpm[ir] * tw;
-                            a_ps += sv * wps[ir] * tw;
-                            a_tm += sv * pw * wtm[ik + koff];
-                            a_ts += sv * pw * wts[ik + koff];
-                        }
+                        *reinterpret_cast<float4*>(row + 4 * (e - (nt + 1))) = make_float4(wn, wm, ws, 0.f);
                     }
-                    __syncwarp(gmask);
                 }
+                __syncwarp(gmask);
+                if (vec4) {
+                    // (row, 4-tick group) items, one 16-byte load of dL/dS each
+                    const float inv_nq = rcp_approx((float)nq);
+                    const int step_r = (int)(((float)G + 0.5f) * inv_nq), step_q = G - step_r * nq;
+                    int ir = (int)(((float)gl + 0.5f) * inv_nq), iq = gl - ir * nq;
+                    const float* tile = dgrid + (int64_t)r0 * c.n_ticks + 4 * q_lo;
+#pragma unroll 1
+                    while (ir < nr) {
+                        const float4 sv = __ldg(reinterpret_cast<const float4*>(
+                            tile + (int64_t)ir * c.n_ticks + 4 * iq));
+                        const float4* q4 = reinterpret_cast<const float4*>(quad + kAdjointQuad * iq);
+                        const float4 w4 = q4[0], m4 = q4[1], g4 = q4[2];
+                        const float4 rw = *reinterpret_cast<const float4*>(row + 4 * ir);
+                        const float A = sv.x * w4.x + sv.y * w4.y + sv.z * w4.z + sv.w * w4.w;
+                        const float B = sv.x * m4.x + sv.y * m4.y + sv.z * m4.z + sv.w * m4.w;
+                        const float C = sv.x * g4.x + sv.y * g4.y + sv.z * g4.z + sv.w * g4.w;
+                        a_q += rw.x * A;
+                        a_pm += rw.y * A;
+                        a_ps += rw.z * A;
+                        a_tm += rw.x * B;
+                        a_ts += rw.x * C;
+                        ir += step_r;
+                        iq += step_q;
+                        if (iq >= nq) { iq -= nq; ++ir; }
+                    }
+                } else {
+                    const float inv_nt = 1.0f / (float)nt;
+                    for (int b = gl; b < nr * nt; b += G) {
+                        const int ir = (int)(((float)b + 0.5f) * inv_nt);
+                        const int ik = b - ir * nt, p = ik + koff;
+                        const float sv = __ldg(dgrid + (int64_t)(r0 + ir) * c.n_ticks + (k0 + ik));
+                        const float* q = quad + (p >> 2) * kAdjointQuad + (p & 3);
+                        const float pw = row[4 * ir], tw = q[0];
+                        a_q += sv * pw * tw;
+                        a_pm += sv * row[4 * ir + 1] * tw;
+                        a_ps += sv * row[4 * ir + 2] * tw;
+                        a_tm += sv * pw * q[4];
+                        a_ts += sv * pw * q[8];
+                    }
+                }
+                __syncwarp(gmask);
             }
-            a_q = group_sum<G>(a_q, gmask);
-            a_pm = group_sum<G>(a_pm, gmask);
-            a_ps = group_sum<G>(a_ps, gmask);
-            a_tm = group_sum<G>(a_tm, gmask);
-            a_ts = group_sum<G>(a_ts, gmask);
         }
+        a_q = group_sum<G>(a_q, gmask);
+        a_pm = group_sum<G>(a_pm, gmask);
+        a_ps = group_sum<G>(a_ps, gmask);
+        a_tm = group_sum<G>(a_tm, gmask);
+        a_ts = group_sum<G>(a_ts, gmask);
         if (gl == 0) {
-            const float qa = dd.ok ? dd.qatt : 0.0f;
-            const float att = (dd.ok && qa > 0.0f) ? qa / d.q[gi] : 0.0f;
+            const float qa = pd.qatt;
             const float dst = qa * a_ps, dsl = qa * a_ts * c.inv_v;
-            if (g.dq) g.dq[gi] = a_q * att;
+            if (g.dq) g.dq[gi] = a_q * pd.att;
             if (g.dp) g.dp[gi] = qa * a_pm;
             if (g.dt) g.dt[gi] = qa * a_tm;
             if (g.dsl) g.dsl[gi] = dsl;
             if (g.dst) g.dst[gi] = dst;
-            if (dd.ok && qa > 0.0f) {
-                s_gt[i][0] = dsl;
-                s_gt[i][1] = dd.st;
-                s_gt[i][2] = dst;
-                s_gt[i][3] = dd.sp;
-                s_gt[i][4] = a_q;
-                s_gt[i][5] = qa;
-            }
+            pd.a_q = a_q;
+            pd.dsl = dsl;
+            pd.dst = dst;
         }
     }
+    if (!g.dglobal) return;
     __syncthreads();
     // The global sums, by one warp for the whole block (FP64 is scarce on this part: one
     // warp instruction per 32 depos).  sigma = sqrt(2 D t_d) gives dsigma/dD = sigma / (2 D)
     // (sigma_L = v sigma_t in mm); dQ'/dtau = Q' t_d / tau^2.  Products of two FP32 values
     // are exact in FP64.
-    if (warp == 0 && g.dglobal) {
+    if (warp == 0) {
         double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-        for (int i = lane; i < kDepos; i += 32) {
-            if (!(s_gt[i][5] > 0.0f)) continue;
-            a0 += (double)s_gt[i][0] * (double)s_gt[i][1];
-            a1 += (double)s_gt[i][2] * (double)s_gt[i][3];
-            a2 += (double)s_gt[i][4] * (double)s_gt[i][5] * d.td[base + i];
+        for (int i = lane; i < kRasterWarps * dpw; i += 32) {
+            const int64_t gi = (int64_t)blockIdx.x * kRasterWarps * dpw + i;
+            const AdjointDepo& p = reinterpret_cast<const AdjointDepo*>(
+                smraw + (i / dpw) * adjoint_warp_smem(dpw))[i % dpw];
+            if (!(p.qatt > 0.0f)) continue;
+            a0 += (double)p.dsl * (double)p.st;
+            a1 += (double)p.dst * (double)p.sp;
+            a2 += (double)p.a_q * (double)p.qatt * d.td[gi];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -784,9 +787,11 @@ cudaError_t launch_depo_adjoint(const RasterConsts& c, const DepoArrays& d, cons
                                 const DepoGrads& g, int* flags, cudaStream_t s)
 {
     if (d.n <= 0) return cudaSuccess;
-    const int64_t blocks = (d.n + kDepos - 1) / kDepos;
-    if (c.renorm) k_depo_adjoint<true><<<(unsigned)blocks, kWarps * 32, 0, s>>>(c, d, dgrid, g, flags);
-    else k_depo_adjoint<false><<<(unsigned)blocks, kWarps * 32, 0, s>>>(c, d, dgrid, g, flags);
+    const int dpw = d.n > 65536 ? 16 : d.n > 16384 ? 8 : 4;
+    const unsigned blocks = (unsigned)rasterize_blocks(d.n, dpw);
+    const int smem = kRasterWarps * adjoint_warp_smem(dpw);
+    if (c.renorm) k_depo_adjoint<true><<<blocks, kRasterWarps * 32, smem, s>>>(c, d, dgrid, g, flags, dpw);
+    else k_depo_adjoint<false><<<blocks, kRasterWarps * 32, smem, s>>>(c, d, dgrid, g, flags, dpw);
     return cudaGetLastError();
 }
 
