@@ -91,6 +91,7 @@ struct wcsim_plane {
     int32_t bclean = 0;         // leading batch grid slots known to be all zero
     int device = 0;
     bool grid_clean = false;    // the plane's grid is all zero (consume-and-clear state)
+    bool after_run = false;     // the last call on the plane was a forward (see launch_chained)
     // wcsim_plane_set_reuse_forward: shat holds the mean-path spectra of the last run on
     // (fwd_depos, fwd_prm) while fwd_valid
     bool reuse_fwd = false;
@@ -198,6 +199,7 @@ RasterConsts make_consts(const wcsim_plane* pl)
     c.renorm = p.renormalize;
     c.keys.set((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
     c.plane_id = p.plane_id;
+    c.chained = 0;
     c.depos_per_block = pl->kd;
     c.lanes_per_depo = pl->kg;
     c.DL = p.DL_cm2_s;
@@ -322,6 +324,23 @@ wcsim_status convolve_stages(wcsim_plane* pl, R2C r2c, float* wave, cudaStream_t
     if ((e = launch_rows_c2r(d, pl->pt, pl->mt, wave, s))) return cuda_fail(e, "rows_c2r launch");
     tl_span(pl, 4, t, tl_record(pl, s));
     return WCSIM_OK;
+}
+
+// Every kernel of this plane's forward is about one wave of CTAs at most.
+bool small_frame(const wcsim_plane* pl)
+{
+    const int64_t wave = 5 * (int64_t)sm_count();
+    const ConvDims& d = pl->dims;
+    return ((int64_t)d.n_w * d.n_imp + 1) / 2 <= wave && 2 * (int64_t)d.nkb <= wave;
+}
+
+// Launches go into a graph: they stay ordinary ones, whose edges any kind of node may end.
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
 }
 
 // A forward that will keep the 2D spectra of S for the backward (set_reuse_forward mode 2):
@@ -633,6 +652,7 @@ wcsim_status wcsim_plane_set_params(wcsim_plane* pl, const wcsim_drift_params* p
     if (!pl) return fail(WCSIM_EINVAL, "plane is NULL");
     wcsim_status st = check_params(params);
     if (st) return st;
+    pl->after_run = false;
     pl->prm = *params;
     return WCSIM_OK;
 }
@@ -643,6 +663,7 @@ wcsim_status wcsim_plane_set_response(wcsim_plane* pl, const void* resp_c64, voi
     if (!resp_c64) return fail(WCSIM_EINVAL, "response pointer is NULL");
     DeviceGuard dg(pl->device);
     if (!dg.ok) return fail(WCSIM_ECUDA, "cannot select the plane's device");
+    pl->after_run = false;
     const ConvDims& d = pl->dims;
     cudaError_t e = launch_make_hermitian(d, (const float2*)resp_c64, pl->H,
                                           (float)(1.0 / ((double)d.n_fw * (double)d.n_ft)),
@@ -713,9 +734,14 @@ static wcsim_status run_frame(wcsim_plane* pl, const wcsim_depos* depos, void* o
         pl->dims.loss = nullptr;
         return st;
     }
+    RasterConsts c = make_consts(pl);
+    pl->dims.chained = pl->after_run && small_frame(pl) && !capturing(s) ? 1 : 0;
+    c.chained = pl->dims.chained && pl->grid_clean && !loss ? 1 : 0;   // no memset of ours before it
+    pl->after_run = false;
     if (!pl->grid_clean) {
         e = cudaMemsetAsync(pl->grid, 0, (size_t)d.n_w * d.n_imp * d.n_t * sizeof(float), s);
         if (e) {
+            pl->dims.chained = 0;
             pl->dims.target = nullptr;
             pl->dims.loss = nullptr;
             return cuda_fail(e, "grid reset");
@@ -723,8 +749,9 @@ static wcsim_status run_frame(wcsim_plane* pl, const wcsim_depos* depos, void* o
     }
     pl->grid_clean = false;
     mark(pl, 1, s);
-    e = launch_rasterize(make_consts(pl), depo_arrays(depos), pl->grid, pl->flags, s);
+    e = launch_rasterize(c, depo_arrays(depos), pl->grid, pl->flags, s);
     if (e) {
+        pl->dims.chained = 0;
         pl->dims.target = nullptr;
         pl->dims.loss = nullptr;
         return cuda_fail(e, "rasterize launch");
@@ -743,12 +770,14 @@ static wcsim_status run_frame(wcsim_plane* pl, const wcsim_depos* depos, void* o
     st = do_convolve(pl, pl->grid, static_cast<float*>(out), s);
     const bool kept = pl->keep_s2d;
     pl->keep_s2d = false;
+    pl->dims.chained = 0;
     pl->dims.clear_input = 0;
     pl->dims.noise_amp = nullptr;
     pl->dims.adc_max = 0;
     pl->dims.target = nullptr;
     pl->dims.loss = nullptr;
     if (st == WCSIM_OK && pl->dims.rows_variant == 0) pl->grid_clean = true;
+    pl->after_run = st == WCSIM_OK;
     if (st == WCSIM_OK && pl->reuse_fwd && pl->prm.fluctuate == 0) {
         pl->fwd_valid = true;           // shat: the mean-path spectra of these depos
         pl->s2d_valid = kept;
@@ -874,6 +903,7 @@ wcsim_status wcsim_run_backward(wcsim_plane* pl, const wcsim_depos* depos, const
                        memcmp(&pl->fwd_depos, depos, sizeof(wcsim_depos)) == 0 &&
                        memcmp(&pl->fwd_prm, &pl->prm, sizeof(wcsim_drift_params)) == 0;
     pl->fwd_valid = false;
+    pl->after_run = false;
     markb(pl, 0, s);
     if (!reuse && !pl->grid_clean) {
         e = cudaMemsetAsync(pl->grid, 0, (size_t)d.n_w * d.n_imp * d.n_t * sizeof(float), s);

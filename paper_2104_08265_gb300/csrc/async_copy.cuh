@@ -16,6 +16,28 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s: far above any legitim
 constexpr int kErrInvalidDepo = 1;                 // device flag bits
 constexpr int kErrTimeout = 2;
 
+// First statement (after work on this CTA's own shared memory and on data that never changes) of
+// every kernel launched with launch_chained, by every thread of it: waits until the kernel before
+// it on the stream has completed and its writes are visible, then lets the next one be put on the
+// SMs.  No CTA may leave before it: the next kernel takes this one's completion for that of
+// everything earlier.
+__device__ __forceinline__ void after_previous_kernel()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Loads of what the kernel before this one wrote: ordinary ones, kept behind
+// after_previous_kernel().  The read-only path (__ldg, or a plain read through a const __restrict__
+// pointer) is for data that does not change while a kernel is on the SMs, and the compiler may move
+// such loads across anything.
+__device__ __forceinline__ float2 ld_fresh(const float2* p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "async_copy.cuh"
 #include "dft_roots.cuh"
 #include "rng.cuh"
 #include "wcsim_internal.cuh"
@@ -366,8 +367,8 @@ __device__ __forceinline__ void stage_herm_pair(const float2* __restrict__ s0,
             const int kk = base + u * blockDim.x;
             a[u] = b[u] = make_float2(0.f, 0.f);
             if (kk < nh) {
-                a[u] = __ldg(s0 + blk_index(kk, w0, n_w));
-                if (has1) b[u] = __ldg(s1 + blk_index(kk, w1, n_w));
+                a[u] = ld_fresh(s0 + blk_index(kk, w0, n_w));
+                if (has1) b[u] = ld_fresh(s1 + blk_index(kk, w1, n_w));
             }
         }
         if (amp) {

@@ -272,6 +272,7 @@ k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __res
                   int pf_ahead, const __grid_constant__ CUtensorMap map, int bk, bool pairs)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
+    after_previous_kernel();
     const int N = p.n;
     float2* X = reinterpret_cast<float2*>(smraw);
     const int64_t n_rows = (int64_t)d.n_w * d.n_imp;
@@ -318,6 +319,7 @@ __global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
 k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
 {
     extern __shared__ __align__(128) unsigned char smraw[];
+    after_previous_kernel();
     mt += blockIdx.y * d.ev_mt;              // event of a batched launch (0 otherwise)
     float* __restrict__ wave = waves.p[blockIdx.y];
     float2* X = reinterpret_cast<float2*>(smraw);
@@ -429,9 +431,10 @@ cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* g
         const size_t sm = row_plan_smem(pt);
         CUtensorMap map;
         const int bk = r2c_store_map(d, pt, shat, 1, &map);
-        k<<<(unsigned)n_pairs, t, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
-                                           r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
-                                           pairs && row_pairs(pt, pt.npass - 1));
+        return launch_chained(d.chained != 0, k, (unsigned)n_pairs, t, sm, s, d, pt,
+                              const_cast<float*>(grid), shat,
+                              r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
+                              pairs && row_pairs(pt, pt.npass - 1));
     }
     return cudaGetLastError();
 }
@@ -453,8 +456,7 @@ cudaError_t launch_rows_c2r_batch(const ConvDims& d, const FftPlan& pt, const fl
     const dim3 grid((unsigned)((d.n_w + 1) / 2), (unsigned)n_ev);
     const int t = row_block(pt, (int64_t)grid.x * grid.y);
     auto k = WCSIM_ROW_KERNEL(k_rows_c2r, row_variant(pt, t));
-    k<<<grid, t, row_plan_smem(pt), s>>>(d, pt, mt, waves);
-    return cudaGetLastError();
+    return launch_chained(d.chained != 0, k, grid, t, row_plan_smem(pt), s, d, pt, mt, waves);
 }
 
 cudaError_t launch_rows_r2c_batch(const ConvDims& d, const FftPlan& pt, const float* grid,
@@ -470,10 +472,9 @@ cudaError_t launch_rows_r2c_batch(const ConvDims& d, const FftPlan& pt, const fl
     const size_t sm = row_plan_smem(pt);
     CUtensorMap map;
     const int bk = r2c_store_map(d, pt, shat, n_ev, &map);
-    k<<<g, t, sm, s>>>(d, pt, const_cast<float*>(grid), shat,
-                       r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
-                                           pairs && row_pairs(pt, pt.npass - 1));
-    return cudaGetLastError();
+    return launch_chained(d.chained != 0, k, g, t, sm, s, d, pt, const_cast<float*>(grid), shat,
+                          r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
+                          pairs && row_pairs(pt, pt.npass - 1));
 }
 
 }  // namespace wcsim

@@ -75,6 +75,7 @@ k_wire_pass(ConvDims d, FftPlan p, const float2* __restrict__ shat, const float2
     const int n_items = my_blocks * d.n_imp;
     const uint32_t bytes_s = (uint32_t)(d.n_w * kBlockCols * sizeof(float2));
     const uint32_t bytes_h = (uint32_t)(N * kBlockCols * sizeof(float2));
+    after_previous_kernel();
 
     auto issue = [&](int i) {           // thread 0: start the copies of item i
         const int kb = blockIdx.x + (i / d.n_imp) * gridDim.x, j = i % d.n_imp, s = i & 1;
@@ -143,7 +144,7 @@ struct BlockedColLd {
     int n_w, kt0;
     __device__ __forceinline__ float2 operator()(int c, int w) const
     {
-        return (w < n_w) ? __ldg(src + blk_index(kt0 + c, w, n_w)) : make_float2(0.f, 0.f);
+        return (w < n_w) ? ld_fresh(src + blk_index(kt0 + c, w, n_w)) : make_float2(0.f, 0.f);
     }
 };
 
@@ -156,6 +157,7 @@ k_wire_direct(ConvDims d, FftPlan p, const float2* __restrict__ shat, const floa
     extern __shared__ __align__(128) unsigned char smraw[];
     const int N = p.n;
     const int plen = padded_len(N) << LG;
+    after_previous_kernel();
     float2* X = reinterpret_cast<float2*>(smraw);
     float2* Y = X + plen;
     float2* acc = Y + plen;
@@ -332,15 +334,14 @@ cudaError_t launch_wire_pass(const ConvDims& d, const FftPlan& pw, const float2*
     const size_t staged = wire_smem_bytes(d.n_w, pw.n);
     if (staged <= kMaxSmem) {
         const int grid = d.nkb < sm_count() ? d.nkb : sm_count();
-        k_wire_pass<<<grid, kThreads, staged, s>>>(d, pw, shat, H, mt, flags);
+        return launch_chained(d.chained != 0, k_wire_pass, grid, kThreads, staged, s, d, pw, shat,
+                              H, mt, flags);
     } else if (3 * (size_t)(padded_len(pw.n) << 2) * sizeof(float2) <= kMaxSmem) {
-        k_wire_direct<2><<<d.nkb, 256, 3 * (size_t)(padded_len(pw.n) << 2) * sizeof(float2), s>>>(
-            d, pw, shat, H, mt);
-    } else {
-        k_wire_direct<0><<<d.nkb * kBlockCols, 256, 3 * (size_t)padded_len(pw.n) * sizeof(float2), s>>>(
-            d, pw, shat, H, mt);
+        return launch_chained(d.chained != 0, k_wire_direct<2>, d.nkb, 256,
+                              3 * (size_t)(padded_len(pw.n) << 2) * sizeof(float2), s, d, pw, shat, H, mt);
     }
-    return cudaGetLastError();
+    return launch_chained(d.chained != 0, k_wire_direct<0>, d.nkb * kBlockCols, 256,
+                          3 * (size_t)padded_len(pw.n) * sizeof(float2), s, d, pw, shat, H, mt);
 }
 
 cudaError_t launch_wire_adjoint_block(const ConvDims& d, const FftPlan& pw, const float2* gt,

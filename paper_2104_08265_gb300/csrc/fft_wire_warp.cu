@@ -69,10 +69,13 @@ k_wire_warp(ConvDims d, const float2* __restrict__ tw2, const float2* __restrict
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
+    }
+    for (int e = threadIdx.x; e < N; e += blockDim.x) s_twf[e] = tw2[e];
+    after_previous_kernel();
+    if (threadIdx.x == 0) {
         mbar_arrive_expect_tx(bar, kTileBytes);
         bulk_g2s(s_h, h_tile(kb), kTileBytes, bar);
     }
-    for (int e = threadIdx.x; e < N; e += blockDim.x) s_twf[e] = tw2[e];
     __syncthreads();
     float2* tr = s_tr[warp];
     float2 acc[32];
@@ -199,18 +202,16 @@ cudaError_t launch_wire_warp(const ConvDims& d, const float2* tw2, const float2*
             attr_set.mark();                                                                   \
         }                                                                                      \
         if (s2d)                                                                               \
-            k_wire_warp<MM, kCols, true><<<grid, kCols * 32, warp_smem<MM, kCols>(), s>>>(     \
-                d, tw2, shat, H, mt, flags, s2d);                                              \
-        else                                                                                   \
-            k_wire_warp<MM, kCols, false><<<grid, kCols * 32, warp_smem<MM, kCols>(), s>>>(    \
-                d, tw2, shat, H, mt, flags, nullptr);                                          \
-        break;                                                                                 \
+            return launch_chained(d.chained != 0, k_wire_warp<MM, kCols, true>, grid,          \
+                                  kCols * 32, warp_smem<MM, kCols>(), s, d, tw2, shat, H, mt,  \
+                                  flags, s2d);                                                 \
+        return launch_chained(d.chained != 0, k_wire_warp<MM, kCols, false>, grid, kCols * 32, \
+                              warp_smem<MM, kCols>(), s, d, tw2, shat, H, mt, flags, s2d);     \
     }
         WCSIM_WARP_M(WCSIM_CASE)
 #undef WCSIM_CASE
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace wcsim

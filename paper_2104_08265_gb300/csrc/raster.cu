@@ -19,6 +19,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "async_copy.cuh"
 #include "binomial.cuh"
 #include "depo_common.cuh"
 #include "rng.cuh"
@@ -377,6 +378,7 @@ k_rasterize(RasterConsts c, DepoArrays d, float* __restrict__ grid, int* flags, 
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ float s_stirl[MODE == 2 ? 16 : 1];
+    after_previous_kernel();
     load_stirling<MODE>(c, s_stirl);
     const int warp = threadIdx.x >> 5;
     rasterize_warp<G, MODE>(c, d, grid, flags, ((int64_t)blockIdx.x * kRasterWarps + warp) * dpw, dpw,
@@ -751,8 +753,9 @@ cudaError_t launch_rasterize(const RasterConsts& c, const DepoArrays& d, float* 
     const unsigned blocks = (unsigned)rasterize_blocks(d.n, t.depos_per_warp);
     const int smem = kRasterWarps * raster_warp_smem(c.fluctuate, t.depos_per_warp, t.lanes_per_depo);
     WCSIM_RASTER_DISPATCH(k_rasterize, t.lanes_per_depo, c.fluctuate,
-        k<<<blocks, kRasterWarps * 32, smem, s>>>(c, d, grid, flags, t.depos_per_warp));
-    return cudaGetLastError();
+        return launch_chained(c.chained != 0, k, blocks, kRasterWarps * 32, smem, s, c, d, grid,
+                              flags, t.depos_per_warp));
+    return cudaSuccess;
 }
 
 cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "async_copy.cuh"
 #include "fft_engine.cuh"
 #include "wcsim_internal.cuh"
 
@@ -78,7 +79,7 @@ __device__ __forceinline__ void load_col(const float2* __restrict__ tile, int c,
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         const int w = lane + 32 * m;
-        v[m] = (w < n_valid) ? __ldg(tile + (int64_t)w * kBlockCols + c) : make_float2(0.f, 0.f);
+        v[m] = (w < n_valid) ? ld_fresh(tile + (int64_t)w * kBlockCols + c) : make_float2(0.f, 0.f);
     }
 }
 

@@ -30,6 +30,7 @@ struct RasterConsts {
     double DL, DT, v, tau;                  // FP64 parameters for the global gradients
     int32_t depos_per_block;                // rasterization tile set by hand or tuned: depos per
     int32_t lanes_per_depo;                 // 8 warps and lanes per depo; 0: by raster_tile
+    int32_t chained;                        // launch_chained of the rasterizer
     float stirl[16];                        // Stirling's remainder log m! - [(m + 1/2) log m
                                             // - m + 1/2 log 2 pi], m = 0..15 (exact binomial)
 };
@@ -152,6 +153,7 @@ struct ConvDims {
     int32_t rows_variant;      // time-axis forward kernel: 0 direct loads, 1 bulk-staged
     int32_t clear_input;       // time-axis forward: write zeros over the rows it has read
     int32_t spectra_tma = 1;   // time-axis kernels: blocked half spectra by TMA box copies
+    int32_t chained = 0;       // launch_chained of the forward's kernels
     int32_t adj_split = 0;     // one-warp wire adjoint: CTAs per frequency block (0: chosen
                                // from the wave fill, adjoint_split)
     // Batched runs: event e's grid, time-axis spectra and wire-summed spectra start
@@ -293,6 +295,32 @@ cudaError_t launch_rows_r2c_fused(const ConvDims& d, const FftPlan& pt, const Ra
 
 // Streaming multiprocessors of the current device (cached).
 int sm_count();
+
+// Launch a kernel that begins with after_previous_kernel().  chained: it may be put on the SMs
+// while the last CTAs of the kernel before it on the stream still run, instead of a launch latency
+// after them.  That pays where a frame is a few short kernels (128 x 1024: 41.8 -> 35.6 us per
+// frame); where kernels fill the SMs for many waves, CTAs that wait there cost more than the
+// latency (960 x 6000 fit step 957 -> 1031 us, a mixed batch 2.87 -> 3.23 ms with every launch
+// chained).  In a torch training loop, which the host bounds, they cost the host more than they
+// give (128 x 1024: 740 -> 780 us per step), so a forward is chained only after another forward.
+template <class... P, class... A>
+cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t s, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, P(args)...);
+    if (e) cudaGetLastError();              // reported here, not by the next check of another call
+    return e;
+}
 
 // A once-per-device flag: kernel attributes (cudaFuncSetAttribute) are set per device, so a
 // process that drives several GPUs sets them once on each.
