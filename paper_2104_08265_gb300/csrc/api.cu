@@ -108,6 +108,7 @@ struct wcsim_plane {
     bool adj_block = false;     // use the block-level wire adjoint even if the warp one fits
     int32_t kd = 0;             // rasterization tile set by hand or by the autotuner: depos per
     int32_t kg = 0;             // 8 warps and lanes per depo (0: chosen per call, raster_tile)
+    int32_t tuned_binomial = -1;    // the tile was tuned with the exact binomial (1), without (0)
     // forward with rasterization fused into the time-axis transform: depo binning scratch,
     // and the impact positions per wire-pass launch (the time-axis spectra of that many
     // impact positions are alive at a time)
@@ -174,6 +175,13 @@ wcsim_status check_depos(const wcsim_depos* d)
 // The per-call constants of the bin decision, in the same operation order the oracle
 // documents: d = pitch / n_imp, 1/d, 1/tick in FP64; 2 D [mm^2/us] = 2 (D 1e-4) rounded to
 // FP32; 1/v, n_sigma, 1/bin rounded to FP32.
+// A tile tuned without the exact binomial is not one for it, nor the other way round (100k depos,
+// binomial: 1196 us by the rule, 1333 with the 8 x 8 tile that the normal mode tunes to).
+bool tile_applies(const wcsim_plane* pl)
+{
+    return pl->tuned_binomial < 0 || pl->tuned_binomial == (pl->prm.fluctuate == 2);
+}
+
 RasterConsts make_consts(const wcsim_plane* pl)
 {
     RasterConsts c;
@@ -200,8 +208,8 @@ RasterConsts make_consts(const wcsim_plane* pl)
     c.keys.set((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
     c.plane_id = p.plane_id;
     c.chained = 0;
-    c.depos_per_block = pl->kd;
-    c.lanes_per_depo = pl->kg;
+    c.depos_per_block = tile_applies(pl) ? pl->kd : 0;
+    c.lanes_per_depo = tile_applies(pl) ? pl->kg : 0;
     c.DL = p.DL_cm2_s;
     c.DT = p.DT_cm2_s;
     c.v = p.v_mm_per_us;
@@ -983,7 +991,8 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
     const RasterConsts c0 = make_consts(planes[0]);
     for (int i = 1; i < n_events && queue; ++i) {
         const wcsim_plane* p = planes[i];
-        queue = p->kd == planes[0]->kd && p->kg == planes[0]->kg &&
+        const bool own = tile_applies(p);
+        queue = (own ? p->kd : 0) == c0.depos_per_block && (own ? p->kg : 0) == c0.lanes_per_depo &&
                 p->prm.fluctuate == c0.fluctuate;
     }
     if (queue) {
@@ -1058,6 +1067,7 @@ wcsim_status wcsim_plane_autotune(wcsim_plane* pl, const wcsim_depos* depos, voi
                                 {256, 16}, {64, 32}, {128, 32}, {256, 32}};    // {0, 0}: the rule
         float best = 1e30f;
         int keep_kd = 0, keep_kg = 0;
+        pl->tuned_binomial = pl->prm.fluctuate == 2;
         for (const auto& t : tiles) {
             pl->kd = t[0];
             pl->kg = t[1];
@@ -1255,6 +1265,7 @@ wcsim_status wcsim_plane_set_raster_tile(wcsim_plane* pl, int32_t depos_per_bloc
                     depos_per_block, lanes_per_depo);
     pl->kd = depos_per_block;
     pl->kg = lanes_per_depo;
+    pl->tuned_binomial = -1;
     return WCSIM_OK;
 }
 

@@ -1,8 +1,9 @@
 // Per-depo drift and bin decision shared by the rasterizers and the adjoint (Sec. 2.1.1
 // "rasterization"; drift and diffusion as in Fig. 2): the FP64 placement of a depo on the
 // impact x tick grid, the FP32 window half-widths, and the FP32 bin masses from erfc edge
-// terms.  Every kernel that rasterizes a depo takes its window and weights from these
-// functions, so that all of them add the same values.
+// terms.  Every kernel that rasterizes a depo takes its window from these functions, so that all
+// of them add to the same bins; the plain rasterizer forms the weights of narrow bins by a series
+// about the bin centres instead, equal to these up to FP32 rounding.
 #pragma once
 
 #include <cuda_runtime.h>

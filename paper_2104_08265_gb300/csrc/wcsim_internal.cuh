@@ -307,6 +307,10 @@ template <class... P, class... A>
 cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
                            cudaStream_t s, A&&... args)
 {
+    if (!chained) {
+        k<<<grid, block, smem, s>>>(P(args)...);
+        return cudaGetLastError();
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -316,7 +320,7 @@ cudaError_t launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block,
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = chained ? 1 : 0;
+    cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k, P(args)...);
     if (e) cudaGetLastError();              // reported here, not by the next check of another call
     return e;
