@@ -60,7 +60,8 @@ __device__ __forceinline__ float binomial_bin(const RasterConsts& c, float qatt,
 // What the lanes of a group need of one depo, formed once by the lane that decides it.  Bin edge e
 // of the window (e bins above its first) lies at u = ((off + e) - frac) s, off the window's first
 // bin relative to the floor of the position (exact in FP32 below 2^24 bins).  A point (sigma == 0,
-// all weight in the window's one bin) has its edges far out on either side.
+// all weight in the window's one bin) has its edges far out on either side of that bin's centre: the
+// bin is the next one (off == 1) for a position so little below an edge that frac rounds up to 1.
 //
 // Bin masses come in two forms.  In general they are differences of erfc at the edges.  Where the
 // bins are not wide against sigma, the mass about a bin's centre c (in units of sqrt(2) sigma,
@@ -92,11 +93,12 @@ __device__ __forceinline__ float offset_float(int64_t k)
     return (int64_t)k32 == k ? (float)k32 : (float)k;
 }
 
-__device__ __forceinline__ void edge_axis(float sigma, float bin, float frac, float& f, float& s)
+__device__ __forceinline__ void edge_axis(float sigma, float bin, float off, float frac, float& f,
+                                          float& s)
 {
     const bool point = !(sigma > 0.0f);
     s = point ? 1e30f : bin / (1.41421356237309505f * sigma);
-    f = point ? 0.5f : frac;
+    f = point ? off + 0.5f : frac;
 }
 
 // Series terms of one axis: term[0] = erf(s / 2), the mass of a bin about the mean, to which the
@@ -152,8 +154,8 @@ __device__ __forceinline__ void make_patch(const RasterConsts& c, const Decision
     p.nt = r.k_hi - r.k_lo + 1;
     p.off_p = offset_float((int64_t)r.r_lo - r.i0p);
     p.off_t = offset_float((int64_t)r.k_lo - r.i0t);
-    edge_axis(r.sp, c.dp_f, r.frac_p, p.frac_p, p.s_p);
-    edge_axis(r.st, c.dt_f, r.frac_t, p.frac_t, p.s_t);
+    edge_axis(r.sp, c.dp_f, p.off_p, r.frac_p, p.frac_p, p.s_p);
+    edge_axis(r.st, c.dt_f, p.off_t, r.frac_t, p.frac_t, p.s_t);
     p.qw = r.qw;
     p.qatt = r.qatt;
     p.inv_q = 1.0f / r.qatt;
@@ -521,8 +523,8 @@ k_depo_adjoint(RasterConsts c, DepoArrays d, const float* __restrict__ dgrid, De
                 p.nt = r.k_hi - r.k_lo + 1;
                 p.off_p = offset_float((int64_t)r.r_lo - r.i0p);
                 p.off_t = offset_float((int64_t)r.k_lo - r.i0t);
-                edge_axis(r.sp, c.dp_f, r.frac_p, p.frac_p, p.s_p);
-                edge_axis(r.st, c.dt_f, r.frac_t, p.frac_t, p.s_t);
+                edge_axis(r.sp, c.dp_f, p.off_p, r.frac_p, p.frac_p, p.s_p);
+                edge_axis(r.st, c.dt_f, p.off_t, r.frac_t, p.frac_t, p.s_t);
                 p.isp = (r.sp > 0.0f) ? 1.0f / r.sp : 0.0f;
                 p.ist = (r.st > 0.0f) ? 1.0f / r.st : 0.0f;
                 p.qatt = r.qatt;
