@@ -321,8 +321,11 @@ k_rows_r2c_fused(ConvDims d, FftPlan p, RasterConsts c, FusedBins b, float2* __r
             float v[4] = {wr * wt.x, wr * wt.y, wr * wt.z, wr * wt.w};
             if (c.fluctuate == 1) {
                 // normal approximation to Binomial(Q', mean / Q'); zero-mean bins stay zero
-                fluctuate4(philox_rounds<0>(make_uint4((uint32_t)q, (uint32_t)(row ? r1 : r0),
-                                                       s_id[h], c.plane_id), c.keys), s_invq[h], v);
+                const uint4 x = philox_rounds<0>(make_uint4((uint32_t)q, (uint32_t)(row ? r1 : r0),
+                                                            s_id[h], c.plane_id), c.keys);
+                const float inv_q = s_invq[h];
+                if (fluctuate_fast(inv_q)) fluctuate4<true>(x, inv_q, v);
+                else fluctuate4<false>(x, inv_q, v);
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e)

@@ -19,6 +19,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "async_copy.cuh"
 #include "binomial.cuh"
 #include "depo_common.cuh"
@@ -325,36 +327,40 @@ __device__ __forceinline__ void rasterize_warp(const RasterConsts& c, const Depo
                 // G / nq and G mod nq (no division per item)
                 const float inv_nq = rcp_approx((float)nq);
                 const int step_r = (int)(((float)G + 0.5f) * inv_nq), step_q = G - step_r * nq;
-                int ir = (int)(((float)gl + 0.5f) * inv_nq), iq = gl - ir * nq;
                 float* tile = grid + (int64_t)r0 * c.n_ticks + 4 * q_lo;
+                auto items = [&](auto fast) {
+                    int ir = (int)(((float)gl + 0.5f) * inv_nq), iq = gl - ir * nq;
 #pragma unroll 1
-                while (ir < nr) {
-                    const float4 t4 = *reinterpret_cast<const float4*>(quad + L::kQuad * iq);
-                    float v[4];
-                    if constexpr (MODE == 1) {
-                        // normal approximation to Binomial(Q', mean / Q'); zero-mean bins
-                        // (outside the window) stay zero
-                        const float4 rr = *reinterpret_cast<const float4*>(row + 4 * ir);
-                        const uint4 qq = *reinterpret_cast<const uint4*>(quad + 8 * iq + 4);
-                        v[0] = rr.x * t4.x; v[1] = rr.x * t4.y; v[2] = rr.x * t4.z; v[3] = rr.x * t4.w;
-                        fluctuate4(philox_rest(qq, __float_as_uint(rr.y), __float_as_uint(rr.z),
-                                               c.keys), inv_q, v);
-                    } else {
-                        const float w = row[ir];
-                        v[0] = w * t4.x; v[1] = w * t4.y; v[2] = w * t4.z; v[3] = w * t4.w;
-                    }
-                    float* dst = tile + (int64_t)ir * c.n_ticks + 4 * iq;
-                    if (vec4) {
-                        atomicAdd(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
-                    } else {
+                    while (ir < nr) {
+                        const float4 t4 = *reinterpret_cast<const float4*>(quad + L::kQuad * iq);
+                        float v[4];
+                        if constexpr (MODE == 1) {
+                            // normal approximation to Binomial(Q', mean / Q'); zero-mean bins
+                            // (outside the window) stay zero
+                            const float4 rr = *reinterpret_cast<const float4*>(row + 4 * ir);
+                            const uint4 qq = *reinterpret_cast<const uint4*>(quad + 8 * iq + 4);
+                            v[0] = rr.x * t4.x; v[1] = rr.x * t4.y; v[2] = rr.x * t4.z; v[3] = rr.x * t4.w;
+                            fluctuate4<decltype(fast)::value>(
+                                philox_rest(qq, __float_as_uint(rr.y), __float_as_uint(rr.z), c.keys), inv_q, v);
+                        } else {
+                            const float w = row[ir];
+                            v[0] = w * t4.x; v[1] = w * t4.y; v[2] = w * t4.z; v[3] = w * t4.w;
+                        }
+                        float* dst = tile + (int64_t)ir * c.n_ticks + 4 * iq;
+                        if (vec4) {
+                            atomicAdd(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
+                        } else {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if ((unsigned)(4 * iq + e - koff) < (unsigned)nt) atomicAdd(dst + e, v[e]);
+                            for (int e = 0; e < 4; ++e)
+                                if ((unsigned)(4 * iq + e - koff) < (unsigned)nt) atomicAdd(dst + e, v[e]);
+                        }
+                        ir += step_r;
+                        iq += step_q;
+                        if (iq >= nq) { iq -= nq; ++ir; }
                     }
-                    ir += step_r;
-                    iq += step_q;
-                    if (iq >= nq) { iq -= nq; ++ir; }
-                }
+                };
+                if (MODE != 1 || fluctuate_fast(inv_q)) items(std::true_type{});
+                else if constexpr (MODE == 1) items(std::false_type{});
                 __syncwarp(gmask);
             }
         }

@@ -108,7 +108,9 @@ __device__ __forceinline__ void box_muller_polar(uint32_t x0, uint32_t x1, float
     const float sc = 2.3283064365386963e-10f, off = 1.1641532182693481e-10f;   // 2^-32, 2^-33
     const float ln2x2 = -1.38629436111989061f;                                 // -2 ln 2
     const float two_pi = 6.28318530717958648f;
-    r2 = ln2x2 * lg2_ftz(fmaf((float)x0, sc, off));       // u0 <= 1: r2 >= 0
+    // u0 <= 1, and lg2.approx.ftz gives no value above 0 for any float of [0.5, 1] (all 2^23 + 1 tried):
+    // r2 >= 0
+    r2 = ln2x2 * lg2_ftz(fmaf((float)x0, sc, off));
     sincos_ftz(fmaf((float)x1, two_pi * sc, two_pi * (off - 0.5f)), sn, cs);
     cs = -cs;
     sn = -sn;
@@ -133,10 +135,25 @@ __device__ __forceinline__ void box_muller4(uint4 x, float z[4])
 }
 
 // The normal approximation to Binomial(Q', v / Q') on four bins of mean v: v + sqrt(v (1 - v / Q'))
-// z, at least 0, with z the four normals of the Philox block x.  The square roots of the
-// variance and of the pair's r2 are taken as one; zero-mean bins stay zero.
+// z, at least 0, with z the four normals of the Philox block x; zero-mean bins stay zero.
+// FAST: the square roots of the variance and of the pair's r2 are taken as one.  Their product (r2
+// is at most 44.4) overflows from Q' = 2^122 on, and the .ftz forms lose it where Q' is small to
+// nothing, so that form is for charges that fluctuate_fast accepts.
+__device__ __forceinline__ bool fluctuate_fast(float inv_q)
+{
+    return inv_q > 0x1p-118f && inv_q < 0x1p80f;
+}
+template <bool FAST>
 __device__ __forceinline__ void fluctuate4(uint4 x, float inv_q, float (&v)[4])
 {
+    if constexpr (!FAST) {
+        float z[4];
+        box_muller4(x, z);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            v[e] = fmaxf(0.0f, fmaf(sqrt_fast(v[e] * (1.0f - v[e] * inv_q)), z[e], v[e]));
+        return;
+    }
     float r2[2], cs[4];
     box_muller_polar(x.x, x.y, r2[0], cs[0], cs[1]);
     box_muller_polar(x.z, x.w, r2[1], cs[2], cs[3]);
