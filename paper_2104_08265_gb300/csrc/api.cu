@@ -82,7 +82,6 @@ struct wcsim_plane {
     float adc_gain = 0.0f, adc_pedestal = 0.0f;   // digitizer (adc_max 0: none set)
     int32_t adc_max = 0;
     int* flags = nullptr;       // device flag word
-    int* queue = nullptr;       // work-queue counter of batched rasterizations
     // scratch of batched runs: bcap events' grids, time-axis and wire-summed spectra
     float* bgrid = nullptr;
     float2* bshat = nullptr;
@@ -248,7 +247,6 @@ void plane_free(wcsim_plane* pl)
     cudaFree(pl->s2d);
     cudaFree(pl->noise_amp);
     cudaFree(pl->flags);
-    cudaFree(pl->queue);
     cudaFree(pl->bgrid);
     cudaFree(pl->bshat);
     cudaFree(pl->bmt);
@@ -490,7 +488,7 @@ wcsim_status prepare_group(wcsim_plane* pl, int k, int32_t* clean_after, cudaStr
     return WCSIM_OK;
 }
 
-// The per-plane rasterization of events idx[0..k) (when the batch's queue launch does not
+// The per-plane rasterization of events idx[0..k) (when the batch's one launch does not
 // apply) into their grid slots.
 wcsim_status rasterize_group(wcsim_plane* pl, int k, const int32_t* idx, const wcsim_depos* depos,
                              cudaStream_t s)
@@ -633,7 +631,6 @@ wcsim_status wcsim_plane_create(const wcsim_geometry* geom, const void* resp_c64
     WC_TRY(cudaMalloc(&pl->shat, n_rows * cols * sizeof(float2)), "spectrum allocation");
     WC_TRY(cudaMalloc(&pl->mt, (size_t)d.n_w * cols * sizeof(float2)), "spectrum allocation");
     WC_TRY(cudaMalloc(&pl->flags, sizeof(int)), "flag allocation");
-    WC_TRY(cudaMalloc(&pl->queue, sizeof(int)), "queue counter allocation");
     WC_TRY(cudaMalloc(&pl->fs.cnt, (size_t)(d.n_w + 1) * sizeof(int32_t)), "bin count allocation");
     WC_TRY(cudaMalloc(&pl->fs.off, (size_t)(d.n_w + 2) * sizeof(int32_t)), "bin offset allocation");
     WC_TRY(cudaMemsetAsync(pl->fs.cnt, 0, (size_t)(d.n_w + 1) * sizeof(int32_t), s), "bin count reset");
@@ -984,19 +981,18 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
         wcsim_status st = prepare_group(planes[first[g]], count[g], &clean_after[g], s);
         if (st) return st;
     }
-    // one persistent rasterization over every event of the batch (a work queue of (event,
-    // depo block) items) when the planes share the rasterization tile and the fluctuation mode;
-    // otherwise one launch per plane
-    bool queue = true;
+    // one rasterization over every event of the batch when the planes share the rasterization tile
+    // and the fluctuation mode; otherwise one launch per plane
+    bool together = true;
     const RasterConsts c0 = make_consts(planes[0]);
-    for (int i = 1; i < n_events && queue; ++i) {
+    for (int i = 1; i < n_events && together; ++i) {
         const wcsim_plane* p = planes[i];
         const bool own = tile_applies(p);
-        queue = (own ? p->kd : 0) == c0.depos_per_block && (own ? p->kg : 0) == c0.lanes_per_depo &&
-                p->prm.fluctuate == c0.fluctuate;
+        together = (own ? p->kd : 0) == c0.depos_per_block && (own ? p->kg : 0) == c0.lanes_per_depo &&
+                   p->prm.fluctuate == c0.fluctuate;
     }
-    if (queue) {
-        QueueEvents q;
+    if (together) {
+        BatchPlanes q;
         int64_t n_depos = 0;
         for (int i = 0; i < n_events; ++i) n_depos += depos[i].n;
         const RasterTile tile = raster_tile(c0, n_depos);
@@ -1012,7 +1008,7 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
             q.flags[i] = p->flags;
             q.block_start[i + 1] = q.block_start[i] + rasterize_blocks(depos[i].n, tile.depos_per_warp);
         }
-        cudaError_t e = launch_rasterize_queue(q, tile, planes[0]->queue, s);
+        cudaError_t e = launch_rasterize_events(q, tile, s);
         if (e) return cuda_fail(e, "batch rasterize launch");
     } else {
         for (int g = 0; g < n_groups; ++g) {

@@ -410,30 +410,29 @@ k_rasterize_batch(RasterConsts c, BatchEvents ev, int* flags, int dpw)
                             smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
 }
 
-// Every event of a batch over a work queue: each warp pops (event, piece of dpw depos) items
-// until the queue is empty (events of different planes carry their own constants).
+// Every event of a batch in one launch, each with its plane's own constants.  A warp's share of depos
+// is a piece, a block's worth of pieces one item of block_start, in the events' order.  The constants
+// are read through the event's index, and a round key that the compiler then holds costs a register:
+// formed from the key instead, the kernel keeps 64 registers and 32 warps per SM.  (Warps that popped
+// their pieces from a queue held 96, 20 warps per SM: 16 events of 2000 to 20000 depos on 480 x 2000
+// and 800 x 6000 planes 180 us with fluctuation, this 94; 12 mixed events 349 / 229.)
 template <int G, int MODE>
-__global__ void __launch_bounds__(kRasterWarps * 32)
-k_rasterize_queue(QueueEvents q, int* queue, int dpw)
+__global__ void __launch_bounds__(kRasterWarps * 32, 8)
+k_rasterize_events(const __grid_constant__ BatchPlanes q, int dpw)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ float s_stirl[MODE == 2 ? 16 : 1];
     load_stirling<MODE>(q.c[0], s_stirl);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int total = q.block_start[q.n];
-    for (;;) {
-        int piece = 0;
-        if (lane == 0) piece = atomicAdd(queue, 1);
-        piece = __shfl_sync(0xffffffffu, piece, 0);
-        const int item = piece / kRasterWarps;
-        if (item >= total) break;
-        int e = 0;
-        while (e + 1 < q.n && q.block_start[e + 1] <= item) ++e;
-        rasterize_warp<G, MODE>(q.c[e], q.d[e], q.grid[e], q.flags[e],
-                                (((int64_t)item - q.block_start[e]) * kRasterWarps + piece % kRasterWarps) * dpw,
-                                dpw, smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
-        __syncwarp();                      // the warp's tile is reused by the next item
-    }
+    const int warp = threadIdx.x >> 5;
+    const int64_t piece = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+    const int item = (int)(piece / kRasterWarps);
+    int e = 0;
+    while (e + 1 < q.n && q.block_start[e + 1] <= item) ++e;
+    RasterConsts c = q.c[e];
+    c.keys.set(c.keys.k0[0], c.keys.k1[0]);
+    rasterize_warp<G, MODE>(c, q.d[e], q.grid[e], q.flags[e],
+                            (piece - (int64_t)q.block_start[e] * kRasterWarps) * dpw, dpw,
+                            smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
 }
 
 // Sum over the G lanes of a lane group (mask: the group's lanes), in every lane of it.
@@ -778,20 +777,17 @@ cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
     return cudaGetLastError();
 }
 
-cudaError_t launch_rasterize_queue(const QueueEvents& q, const RasterTile& t, int* queue,
-                                   cudaStream_t s)
+cudaError_t launch_rasterize_events(const BatchPlanes& q, const RasterTile& t, cudaStream_t s)
 {
-    const int total = q.block_start[q.n];
-    if (q.n <= 0 || total <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int), s);
-    if (e) return e;
+    const int blocks = q.n > 0 ? q.block_start[q.n] : 0;
+    if (blocks <= 0) return cudaSuccess;
     const int mode = q.c[0].fluctuate;
-    const int smem = kRasterWarps * raster_warp_smem(mode, t.depos_per_warp, t.lanes_per_depo);
-    WCSIM_RASTER_DISPATCH(k_rasterize_queue, t.lanes_per_depo, mode,
-        int per_sm = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kRasterWarps * 32, smem))) return e;
-        const int resident = (per_sm > 0 ? per_sm : 1) * sm_count();
-        k<<<total < resident ? total : resident, kRasterWarps * 32, smem, s>>>(q, queue, t.depos_per_warp));
+    // one warp per block for the exact binomial, whose walks differ much in length (16 events of 2000
+    // to 20000 depos: 2043 us, with four 2096)
+    const int warps = mode == 2 ? 1 : kRasterWarps;
+    const int smem = warps * raster_warp_smem(mode, t.depos_per_warp, t.lanes_per_depo);
+    WCSIM_RASTER_DISPATCH(k_rasterize_events, t.lanes_per_depo, mode,
+        k<<<(unsigned)blocks * (kRasterWarps / warps), warps * 32, smem, s>>>(q, t.depos_per_warp));
     return cudaGetLastError();
 }
 

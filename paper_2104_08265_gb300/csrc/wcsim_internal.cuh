@@ -60,11 +60,10 @@ struct BatchEvents {
     uint32_t key0[kMaxBatch], key1[kMaxBatch];
 };
 
-// Every event of a batch, whatever its plane, for one persistent rasterization over a work
-// queue of (event, depo block) items; passed by value.
-struct QueueEvents {
+// Every event of a batch, whatever its plane, for one rasterization; passed by value.
+struct BatchPlanes {
     int32_t n;
-    int32_t block_start[kMaxBatch + 1];  // first item of each event (prefix sum)
+    int32_t block_start[kMaxBatch + 1];  // first block of each event (prefix sum)
     RasterConsts c[kMaxBatch];           // the event's plane constants and fluctuation key
     DepoArrays d[kMaxBatch];
     float* grid[kMaxBatch];
@@ -91,11 +90,9 @@ cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
                                    const RasterTile& t, int* flags, cudaStream_t s);
 // CTAs that n_depos depos take.
 int rasterize_blocks(int64_t n_depos, int depos_per_warp);
-// Rasterize every event of q in one persistent launch: warps pop pieces of the events' blocks
-// from *queue (zeroed here on the stream first) until all q.block_start[q.n] are done.  All
-// events use the tile t and the fluctuation mode of q.c[0].
-cudaError_t launch_rasterize_queue(const QueueEvents& q, const RasterTile& t, int* queue,
-                                   cudaStream_t s);
+// Rasterize every event of q in one launch.  All events use the tile t and the fluctuation mode of
+// q.c[0].
+cudaError_t launch_rasterize_events(const BatchPlanes& q, const RasterTile& t, cudaStream_t s);
 // Whether a tile may be set (depos per 8 warps, lanes per depo).
 bool raster_tile_supported(int depos_per_block, int lanes_per_depo);
 // Adjoint of drift + rasterization (mean path, windows fixed): dgrid -> per-depo and global
