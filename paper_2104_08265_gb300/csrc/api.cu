@@ -982,14 +982,15 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
         if (st) return st;
     }
     // one rasterization over every event of the batch when the planes share the rasterization tile
-    // and the fluctuation mode; otherwise one launch per plane
+    // and the kind of fluctuation draw (normal or none, or exact binomial); otherwise one launch per
+    // plane
     bool together = true;
     const RasterConsts c0 = make_consts(planes[0]);
     for (int i = 1; i < n_events && together; ++i) {
         const wcsim_plane* p = planes[i];
         const bool own = tile_applies(p);
         together = (own ? p->kd : 0) == c0.depos_per_block && (own ? p->kg : 0) == c0.lanes_per_depo &&
-                   p->prm.fluctuate == c0.fluctuate;
+                   (p->prm.fluctuate == 2) == (c0.fluctuate == 2);
     }
     if (together) {
         BatchPlanes q;

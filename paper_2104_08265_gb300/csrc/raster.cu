@@ -416,6 +416,8 @@ k_rasterize_batch(RasterConsts c, BatchEvents ev, int* flags, int dpw)
 // formed from the key instead, the kernel keeps 64 registers and 32 warps per SM.  (Warps that popped
 // their pieces from a queue held 96, 20 warps per SM: 16 events of 2000 to 20000 depos on 480 x 2000
 // and 800 x 6000 planes 180 us with fluctuation, this 94; 12 mixed events 349 / 229.)
+// MODE kMixed: events with the normal fluctuation and without.
+constexpr int kMixed = 3;
 template <int G, int MODE>
 __global__ void __launch_bounds__(kRasterWarps * 32, 8)
 k_rasterize_events(const __grid_constant__ BatchPlanes q, int dpw)
@@ -430,9 +432,16 @@ k_rasterize_events(const __grid_constant__ BatchPlanes q, int dpw)
     while (e + 1 < q.n && q.block_start[e + 1] <= item) ++e;
     RasterConsts c = q.c[e];
     c.keys.set(c.keys.k0[0], c.keys.k1[0]);
-    rasterize_warp<G, MODE>(c, q.d[e], q.grid[e], q.flags[e],
-                            (piece - (int64_t)q.block_start[e] * kRasterWarps) * dpw, dpw,
-                            smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
+    const int64_t base = (piece - (int64_t)q.block_start[e] * kRasterWarps) * dpw;
+    constexpr int kOne = MODE == kMixed ? 1 : MODE;
+    unsigned char* tile = smraw + warp * raster_warp_smem(kOne, dpw, G);
+    if constexpr (MODE == kMixed) {
+        if (c.fluctuate == 0) {
+            rasterize_warp<G, 0>(c, q.d[e], q.grid[e], q.flags[e], base, dpw, tile, s_stirl);
+            return;
+        }
+    }
+    rasterize_warp<G, kOne>(c, q.d[e], q.grid[e], q.flags[e], base, dpw, tile, s_stirl);
 }
 
 // Sum over the G lanes of a lane group (mask: the group's lanes), in every lane of it.
@@ -782,6 +791,15 @@ cudaError_t launch_rasterize_events(const BatchPlanes& q, const RasterTile& t, c
     const int blocks = q.n > 0 ? q.block_start[q.n] : 0;
     if (blocks <= 0) return cudaSuccess;
     const int mode = q.c[0].fluctuate;
+    for (int e = 1; e < q.n; ++e) {
+        if (q.c[e].fluctuate == mode) continue;
+        if (mode == 2 || q.c[e].fluctuate == 2) return cudaErrorInvalidValue;
+        auto k = t.lanes_per_depo == 8 ? k_rasterize_events<8, kMixed>
+                 : t.lanes_per_depo == 16 ? k_rasterize_events<16, kMixed> : k_rasterize_events<32, kMixed>;
+        k<<<(unsigned)blocks, kRasterWarps * 32,
+            kRasterWarps * raster_warp_smem(1, t.depos_per_warp, t.lanes_per_depo), s>>>(q, t.depos_per_warp);
+        return cudaGetLastError();
+    }
     // one warp per block for the exact binomial, whose walks differ much in length (16 events of 2000
     // to 20000 depos: 2043 us, with four 2096)
     const int warps = mode == 2 ? 1 : kRasterWarps;

@@ -90,8 +90,8 @@ cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
                                    const RasterTile& t, int* flags, cudaStream_t s);
 // CTAs that n_depos depos take.
 int rasterize_blocks(int64_t n_depos, int depos_per_warp);
-// Rasterize every event of q in one launch.  All events use the tile t and the fluctuation mode of
-// q.c[0].
+// Rasterize every event of q in one launch with the tile t.  Events with the normal fluctuation and
+// without share it, the exact binomial (fluctuate == 2) has its own.
 cudaError_t launch_rasterize_events(const BatchPlanes& q, const RasterTile& t, cudaStream_t s);
 // Whether a tile may be set (depos per 8 warps, lanes per depo).
 bool raster_tile_supported(int depos_per_block, int lanes_per_depo);
