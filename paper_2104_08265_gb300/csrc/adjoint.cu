@@ -164,7 +164,8 @@ k_wire_adjoint_b(ConvDims d, const float2* __restrict__ tw2, const float2* __res
     }
 }
 
-template <int V>
+// V, pairs: row_launch (kRow6000 has an instance each for pairs, PAIRS, and without).
+template <int V, bool PAIRS = true>
 __global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
 k_rows_c2r_grid(ConvDims d, FftPlan p, const float2* __restrict__ shat, float* __restrict__ grid,
                 bool pairs)
@@ -177,17 +178,28 @@ k_rows_c2r_grid(ConvDims d, FftPlan p, const float2* __restrict__ shat, float* _
     const int j = blockIdx.x / npw, w0 = 2 * (blockIdx.x % npw), w1 = w0 + 1;
     const bool has1 = w1 < d.n_w;
     const int64_t slab = (int64_t)d.nkb * d.n_w * kBlockCols;
-    if (pairs) {
-        run_row_inverse_pairs<V>(p, X, shat + j * slab, w0, has1, d.n_w);
-    } else {
+    constexpr bool PAD = V == kRowTwo;
+    const float2* z = X;
+    auto stage = [&] {
         stage_herm_pair(shat + j * slab, shat + j * slab, w0, has1 ? w1 : w0, has1, d.n_w, d.nh, p.n, X);
         __syncthreads();
-        run_row_inverse<V>(p, X);
+    };
+    if constexpr (V == kRowTwo) {
+        stage();
+        z = run_plan<true, 0>(p, FlatLd<0>{X}, X + padded_len(p.n), X);
+    } else {
+        if constexpr (V == kRow6000) pairs = PAIRS;
+        if (pairs) {
+            run_row_inverse_pairs<V>(p, X, shat + j * slab, w0, has1, d.n_w);
+        } else {
+            stage();
+            run_row_inverse<V>(p, X);
+        }
     }
     float* o0 = grid + ((int64_t)w0 * d.n_imp + j) * d.n_t;
     float* o1 = grid + ((int64_t)w1 * d.n_imp + j) * d.n_t;
     const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(grid) & 7) == 0);
-    store_real_pair(X, o0, o1, d.n_t, has1, vec);
+    store_real_pair<PAD>(z, o0, o1, d.n_t, has1, vec);
 }
 
 // dL/dR_j(kw, kt) = conj(S_j^(kw, kt)) G^(kw, kt) / n and its Hermitian mirror (-kw, -kt)
@@ -325,15 +337,17 @@ cudaError_t launch_rows_c2r_grid(const ConvDims& d, const FftPlan& pt, const flo
         for (int v = 0; v < kRowVariants && !e; ++v)
             e = cudaFuncSetAttribute(WCSIM_ROW_KERNEL(k_rows_c2r_grid, v),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (!e) e = cudaFuncSetAttribute(k_rows_c2r_grid<kRow6000, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e) return e;
         g_attr.mark();
     }
     const int64_t n_ctas = (int64_t)d.n_imp * ((d.n_w + 1) / 2);
-    const int t = row_block(pt, n_ctas);
-    auto k = WCSIM_ROW_KERNEL(k_rows_c2r_grid, row_variant(pt, t));
     // mirrored pairs (run_row_inverse_pairs) from a few waves up
-    const bool pairs = row_pairs(pt, 0) && n_ctas > 8 * sm_count();
-    k<<<(unsigned)n_ctas, t, row_plan_smem(pt), s>>>(d, pt, shat, grid, pairs);
+    const RowLaunch l = row_launch(pt, n_ctas, kRowGrid, n_ctas > 8 * sm_count());
+    auto k = l.variant == kRow6000 && !l.pairs ? k_rows_c2r_grid<kRow6000, false>
+                                               : WCSIM_ROW_KERNEL(k_rows_c2r_grid, l.variant);
+    k<<<(unsigned)n_ctas, l.threads, l.smem, s>>>(d, pt, shat, grid, l.pairs);
     return cudaGetLastError();
 }
 

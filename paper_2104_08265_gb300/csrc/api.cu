@@ -842,7 +842,7 @@ static wcsim_status convolve_adjoint(wcsim_plane* pl, const float* grad_wave, co
     if (!have_shat && (e = launch_rows_r2c(d, pl->pt, grid, pl->shat, pl->flags, s)))
         return cuda_fail(e, "rows_r2c launch");
     markb(pl, 3, s);
-    if ((e = launch_rows_r2c(dG, pl->pt, grad_wave, pl->mt, pl->flags, s, false))) return cuda_fail(e, "rows_r2c launch");
+    if ((e = launch_rows_r2c(dG, pl->pt, grad_wave, pl->mt, pl->flags, s, &d))) return cuda_fail(e, "rows_r2c launch");
     markb(pl, 4, s);
     const float inv_n = (float)(1.0 / ((double)d.n_fw * (double)d.n_ft));
     const bool warp = pl->tw_warp && !pl->adj_block;

@@ -399,11 +399,25 @@ __device__ __forceinline__ void stage_herm_pair(const float2* __restrict__ s0,
     }
 }
 
+// Ticks 2q and 2q + 1 of a transform in z (16-byte aligned); PAD: z is padded (run_plan; the two lie
+// in one group of 16).
+template <bool PAD>
+__device__ __forceinline__ float4 tick_pair(const float2* z, int q)
+{
+    if constexpr (PAD) {
+        const float2 *p = z + pad16(2 * q), a = p[0], b = p[1];
+        return make_float4(a.x, a.y, b.x, b.y);
+    } else {
+        return reinterpret_cast<const float4*>(z)[q];
+    }
+}
+
 // Write the two real rows of an inverse real-pair transform held in z (16-byte aligned; row 0 in
-// .x, row 1 in .y; o1 ignored when !has1), ticks t < n_t.  With vec (rows 8-byte aligned, n_t
-// even) a thread takes 2 ticks: consecutive lanes read consecutive 16 bytes of shared memory, free
-// of bank conflicts, and write 8 bytes of each row (four ticks per thread, with 16-byte stores,
-// read 32 bytes apart: the inverse FFT of dL/dS took 144 us with it).
+// .x, row 1 in .y; o1 ignored when !has1; PAD: z is padded), ticks t < n_t.  With vec (rows 8-byte
+// aligned, n_t even) a thread takes 2 ticks: consecutive lanes read consecutive 16 bytes of shared
+// memory, free of bank conflicts, and write 8 bytes of each row (four ticks per thread, with 16-byte
+// stores, read 32 bytes apart: the inverse FFT of dL/dS took 144 us with it).
+template <bool PAD>
 __device__ __forceinline__ void store_real_pair(const float2* z, float* __restrict__ o0,
                                                 float* __restrict__ o1, int n_t, bool has1,
                                                 bool vec)
@@ -412,13 +426,13 @@ __device__ __forceinline__ void store_real_pair(const float2* z, float* __restri
         float2* p0 = reinterpret_cast<float2*>(o0);
         float2* p1 = reinterpret_cast<float2*>(o1);
         for (int q = threadIdx.x; q < (n_t >> 1); q += blockDim.x) {
-            const float4 a = reinterpret_cast<const float4*>(z)[q];       // ticks 2q, 2q + 1
+            const float4 a = tick_pair<PAD>(z, q);
             p0[q] = make_float2(a.x, a.z);
             if (has1) p1[q] = make_float2(a.y, a.w);
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[t];
+            const float2 v = z[PAD ? pad16(t) : t];
             o0[t] = v.x;
             if (has1) o1[t] = v.y;
         }
@@ -429,6 +443,7 @@ __device__ __forceinline__ void store_real_pair(const float2* z, float* __restri
 // store_real_pair would write) for rows 0 (.x, target t0) and 1 (.y, t1); returns this
 // thread's FP32 sum of the squared residuals it wrote.  vec: rows and targets 8-byte aligned,
 // n_t even.
+template <bool PAD>
 __device__ __forceinline__ float store_residual_pair(const float2* z, float* __restrict__ o0,
                                                     float* __restrict__ o1,
                                                     const float* __restrict__ t0,
@@ -456,7 +471,7 @@ __device__ __forceinline__ float store_residual_pair(const float2* z, float* __r
             for (int u = 0; u < kU; ++u) {
                 const int q = base + u * blockDim.x;
                 if (q < nq) {
-                    const float4 a = reinterpret_cast<const float4*>(z)[q];
+                    const float4 a = tick_pair<PAD>(z, q);
                     const float2 r0 = make_float2(__fsub_rn(a.x, ta[u].x), __fsub_rn(a.z, ta[u].y));
                     reinterpret_cast<float2*>(o0)[q] = r0;
                     ss += r0.x * r0.x + r0.y * r0.y;
@@ -470,7 +485,7 @@ __device__ __forceinline__ float store_residual_pair(const float2* z, float* __r
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[t];
+            const float2 v = z[PAD ? pad16(t) : t];
             const float r0 = __fsub_rn(v.x, t0[t]);
             o0[t] = r0;
             ss += r0 * r0;
@@ -495,6 +510,7 @@ __device__ __forceinline__ uint16_t adc_code(float m, float g, float p, float to
 
 // store_real_pair for ADC codes: row 0 (.x) to o0, row 1 (.y) to o1, uint16.  With vec (rows
 // 4-byte aligned, n_t even) a thread writes 2 codes per row with one 4-byte store.
+template <bool PAD>
 __device__ __forceinline__ void store_real_pair_adc(const float2* z, uint16_t* __restrict__ o0,
                                                     uint16_t* __restrict__ o1, int n_t, bool has1,
                                                     bool vec, float g, float p, float top)
@@ -506,13 +522,13 @@ __device__ __forceinline__ void store_real_pair_adc(const float2* z, uint16_t* _
             return (uint32_t)adc_code(u, g, p, top) | ((uint32_t)adc_code(v, g, p, top) << 16);
         };
         for (int q = threadIdx.x; q < (n_t >> 1); q += blockDim.x) {
-            const float4 a = reinterpret_cast<const float4*>(z)[q];
+            const float4 a = tick_pair<PAD>(z, q);
             p0[q] = pack(a.x, a.z);
             if (has1) p1[q] = pack(a.y, a.w);
         }
     } else {
         for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
-            const float2 v = z[t];
+            const float2 v = z[PAD ? pad16(t) : t];
             o0[t] = adc_code(v.x, g, p, top);
             if (has1) o1[t] = adc_code(v.y, g, p, top);
         }
@@ -822,19 +838,21 @@ __host__ inline int row_threads(const FftPlan& p)
     return (t + 31) & ~31;
 }
 
-// Row-kernel instances: the compile-time 6000-point plan (radices 16, 25, 15; 256 threads), and
-// the runtime plan for blocks of up to so many threads.  All keep one padded buffer per CTA and
-// 72 to 80 registers per thread (96 for the largest), so registers and shared memory give out
-// together: 24 warps per SM at 6000 points, 26 at 9600, where two ping-pong buffers of the same
-// plan left 8 to 16.
-enum RowVariant : int { kRow6000 = 0, kRow128, kRow256, kRow448, kRow704, kRowVariants };
+// Row-kernel instances: the compile-time 6000-point plan (radices 16, 25, 15; 256 threads); the
+// runtime plan in place, for blocks of up to 384, 448 and 704 threads; and the runtime plan between
+// two buffers (run_plan, 256 threads).  The in-place ones keep 72 (448) to 80 registers per thread, so
+// that registers and shared memory give out together: 24 warps per SM at 6000 points, 26 at 9600,
+// where two buffers leave 8 to 16.  What they pay for it is code: every pass unrolls the butterflies
+// that a thread holds (the runtime ones spill 48 to 124 bytes per thread, that of 448 threads 192 to
+// 792), and a kernel of one wave or two spends much of its time fetching instructions.
+enum RowVariant : int { kRow6000 = 0, kRow384, kRow448, kRow704, kRowTwo, kRowVariants };
 __host__ __device__ constexpr int row_max_threads(int v)
 {
-    return v == kRow128 ? 128 : v == kRow448 ? 448 : v == kRow704 ? 704 : 256;
+    return v == kRow384 ? 384 : v == kRow448 ? 448 : v == kRow704 ? 704 : 256;
 }
 __host__ __device__ constexpr int row_min_ctas(int v)
 {
-    return v == kRow128 ? 6 : v == kRow448 ? 2 : v == kRow704 ? 1 : 3;
+    return v == kRow6000 ? 3 : v == kRow704 ? 1 : 2;
 }
 
 __host__ inline bool is_plan6000(const FftPlan& p)
@@ -842,22 +860,15 @@ __host__ inline bool is_plan6000(const FftPlan& p)
     return p.n == 6000 && p.npass == 3 && p.radix[0] == 16 && p.radix[1] == 25 && p.radix[2] == 15;
 }
 
-// Block of a row kernel for plan p over `ctas` CTAs: what the plan needs; 256 threads at least when
-// the CTAs are few for the SMs (a short transform's staging and stores are then what a CTA waits
+// Block of an in-place row kernel for plan p over `ctas` CTAs: what the plan needs; 256 threads at least
+// when the CTAs are few for the SMs (a short transform's staging and stores are then what a CTA waits
 // for), or instead of 128 from 3500 points on (9600 rows of 4096 points 134 -> 127 us, 2500 of 3840
 // 53.6 -> 47.9; of 3072 points 94 -> 107, the other way round).
 __host__ inline int row_block(const FftPlan& p, int64_t ctas)
 {
-    if (is_plan6000(p)) return 256;
     const int t = row_threads(p);
     if (t < 256 && (ctas < 4 * (int64_t)sm_count() || (t == 128 && p.n > 3500))) return 256;
     return t;
-}
-
-__host__ inline RowVariant row_variant(const FftPlan& p, int block)
-{
-    if (is_plan6000(p)) return kRow6000;
-    return block <= 128 ? kRow128 : block <= 256 ? kRow256 : block <= 448 ? kRow448 : kRow704;
 }
 
 // Whether pass i of plan p, its first or last, can run on units of two mirrored butterflies: the
@@ -937,8 +948,8 @@ __device__ __forceinline__ void run_row_inverse_pairs(const FftPlan& p, float2* 
     }
 }
 
-// Shared bytes of a row kernel for plan p: n complex values and one pad per even group of the
-// passes' layouts (at least padded_len(n), which the flat rows of the TMA stores are sized to).
+// Shared bytes of an in-place row kernel for plan p: n complex values and one pad per even group of
+// the passes' layouts (at least padded_len(n), which the flat rows of the TMA stores are sized to).
 __host__ inline size_t row_plan_smem(const FftPlan& p)
 {
     int len = padded_len(p.n);
@@ -949,9 +960,62 @@ __host__ inline size_t row_plan_smem(const FftPlan& p)
     return (size_t)len * sizeof(float2);
 }
 
+// How a row transform of plan p over `ctas` CTAs is launched.  pairs: the spectra of S and the inverse
+// of dL/dS may take mirrored butterflies together.
+enum RowUse : int { kRowForward, kRowFrame, kRowGrid };
+struct RowLaunch {
+    RowVariant variant;
+    int threads;
+    size_t smem;
+    bool pairs;
+};
+
+// In place or between two buffers?  In place puts more CTAs on an SM and can pair butterflies; two
+// buffers run a fraction of the code, which a launch of one round or two spends most of its time
+// fetching.  So the rounds that the CTAs take either way decide, up to 6000 points (above 6700 two
+// buffers leave one CTA per SM; between, in place is ahead).  Times between two buffers over times in
+// place, 64 to 960 wires x 10 rows, 512 to 5760 points:
+// - the frame's inverse: 0.75 to 0.97 where two buffers need no more rounds, 1.1 to 1.3 where they do;
+// - spectra of S and inverse of dL/dS: 0.65 to 1.0 where a second round in place is a small one (480
+//   CTAs, at 160 threads 640 to 800), 1.0 to 1.8 else.  Two buffers may take 6/5 the rounds for the
+//   spectra, 8/5 up to 4200 points, 2 from 3000 there without pairs where there is a second round (4000
+//   points, 1280 CTAs: 0.93), and 8/5 for the inverse; from four rounds in place on they never do;
+// - except that passes of radix 16 and more, without pairs, gain nothing in place (4096 points: 0.91 to
+//   0.97 at any size).
+__host__ inline RowLaunch row_launch(const FftPlan& p, int64_t ctas, RowUse use, bool pairs)
+{
+    if (is_plan6000(p)) return {kRow6000, 256, row_plan_smem(p), pairs};
+    pairs = pairs && row_pairs(p, use == kRowForward ? p.npass - 1 : 0);
+    const int t = row_block(p, ctas);
+    const RowVariant v = t <= 384 ? kRow384 : t <= 448 ? kRow448 : kRow704;
+    const size_t one = row_plan_smem(p), two = 2 * (size_t)padded_len(p.n) * sizeof(float2);
+    const size_t sm = 228 * 1024, reserved = 1024;              // shared memory of an SM, and per CTA
+    auto rounds = [&](int per_regs, size_t bytes) {
+        const int64_t fit = (int64_t)(sm / (bytes + reserved));
+        const int64_t per = (fit < per_regs ? (fit > 0 ? fit : 1) : per_regs) * sm_count();
+        return (ctas + per - 1) / per;
+    };
+    // warps per SM by registers: 6 per quarter at 80 registers, 7 at 72
+    const int64_t r1 = rounds((v == kRow448 ? 28 : 24) / (t / 32), one), r2 = rounds(2, two);
+    bool use_two = false;
+    if (use == kRowFrame) {
+        use_two = p.n <= 6000 && r2 <= r1;
+    } else if (p.n <= 6000 && r1 <= 3) {
+        const int fifths = use == kRowGrid ? 8 : p.n > 4200 ? 6 : !pairs && r1 > 1 && p.n > 3000 ? 10 : 8;
+        use_two = 5 * r2 <= fifths * r1;
+    }
+    if (use == kRowForward && !pairs && p.n <= 6700) {
+        bool large = true;
+        for (int i = 0; i < p.npass; ++i) large = large && p.radix[i] >= 16;
+        use_two = use_two || large;
+    }
+    if (use_two) return {kRowTwo, 256, two, false};
+    return {v, t, one, pairs};
+}
+
 // The instance of kernel template K for variant v.
 #define WCSIM_ROW_KERNEL(K, v)                                                                    \
-    ((v) == kRow6000 ? K<kRow6000> : (v) == kRow128 ? K<kRow128> : (v) == kRow256 ? K<kRow256>    \
-     : (v) == kRow448 ? K<kRow448> : K<kRow704>)
+    ((v) == kRow6000 ? K<kRow6000> : (v) == kRow384 ? K<kRow384> : (v) == kRow448 ? K<kRow448>    \
+     : (v) == kRow704 ? K<kRow704> : K<kRowTwo>)
 
 }  // namespace wcsim

@@ -6,8 +6,8 @@
 // rows_r2c (direct, the default) takes one pair of rows per CTA: both rows are loaded into
 // shared memory with batched 16-byte loads (scalar loads when rows are not 16-byte aligned),
 // a pair with no nonzero value stores zero spectra at once, and otherwise every pass of the
-// plan runs in place in one shared buffer; the CTA also asks L2 for the rows of the CTA
-// expected to follow it on the SM.  The two half spectra are separated into flat shared rows
+// plan runs in shared memory, in place or between two buffers (row_launch); the CTA also asks
+// L2 for the rows of the CTA expected to follow it on the SM.  The two half spectra are separated into flat shared rows
 // and leave through TMA tensor box stores (per-thread stores with WCSIM_SPECTRA_TMA=0).
 // rows_r2c (staged, chosen by the autotuner or
 // WCSIM_ROWS_KERNEL) is persistent: one CTA per SM walks pairs of rows, and one bulk copy
@@ -151,32 +151,40 @@ __device__ __forceinline__ float2* align128(float2* p)
 
 // Separate the pair's half spectra as store_pair_spectra does, into flat shared rows for the
 // TMA box stores: row 0's X0[k] at f[k], row 1's X1[k] at f[o1 + k], zeros for nh <= k < nk.
-// f may alias z: every thread first reads its frequencies k = tid + i T, i < NI (NI T >= nh), into
-// registers, the block of T threads synchronises, then writes.  Ends with a proxy fence and a
-// block barrier (the async proxy may then read f).
+// NI > 0: f may alias z (unpadded); every thread of the block of T first reads its frequencies
+// k = tid + i T, i < NI (NI T >= nh), into registers, the block synchronises, then writes.  NI = 0: f
+// and z are distinct buffers, z padded (run_plan).  Ends with a proxy fence and a block barrier (the
+// async proxy may then read f).
 template <int NI>
 __device__ __forceinline__ void separate_flat(const float2* z, int N, int nh, int nk, int o1,
-                                              float2* f)
+                                              float2* f, const int T)
 {
-    const int T = blockDim.x;
-    float2 a0[NI], a1[NI];
+    auto sep = [&](const float2 a, const float2 b, float2& x0, float2& x1) {
+        x0 = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
+        x1 = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+    };
+    if constexpr (NI > 0) {
+        float2 a0[NI], a1[NI];
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-        const int k = threadIdx.x + i * T;
-        if (k < nh) {
-            const float2 a = z[k];
-            const float2 b = z[k == 0 ? 0 : N - k];
-            a0[i] = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-            a1[i] = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+        for (int i = 0; i < NI; ++i) {
+            const int k = threadIdx.x + i * T;
+            if (k < nh) sep(z[k], z[k == 0 ? 0 : N - k], a0[i], a1[i]);
         }
-    }
-    __syncthreads();
+        __syncthreads();
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-        const int k = threadIdx.x + i * T;
-        if (k < nh) {
-            f[k] = a0[i];
-            f[o1 + k] = a1[i];
+        for (int i = 0; i < NI; ++i) {
+            const int k = threadIdx.x + i * T;
+            if (k < nh) {
+                f[k] = a0[i];
+                f[o1 + k] = a1[i];
+            }
+        }
+    } else {
+        for (int k = threadIdx.x; k < nh; k += T) {
+            float2 x0, x1;
+            sep(z[pad16(k)], z[k == 0 ? 0 : pad16(N - k)], x0, x1);
+            f[k] = x0;
+            f[o1 + k] = x1;
         }
     }
     for (int k = nh + threadIdx.x; k < nk; k += T) f[k] = f[o1 + k] = make_float2(0.f, 0.f);
@@ -263,10 +271,10 @@ k_rows_r2c_staged(ConvDims d, FftPlan p, const float* __restrict__ grid, float2*
 
 // pf_ahead > 0: CTA b first asks L2 for the rows of pair b + pf_ahead (the CTA that will
 // most likely take over its slot once it retires), so that pair's first pass reads L2.
-// V: row_variant; pairs: row_pairs of the last pass.
+// V, pairs: row_launch (kRow6000 has an instance each for pairs, PAIRS, and without).
 // bk > 0: the half spectra leave through TMA box stores of bk frequency blocks (map: the
-// blocked spectra, events along its last dimension); bk = 0: plain stores.
-template <int V>
+// blocked spectra, events along its last dimension); bk = 0: plain stores, and no pairs.
+template <int V, bool PAIRS = true>
 __global__ void __launch_bounds__(row_max_threads(V), row_min_ctas(V))
 k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __restrict__ shat,
                   int pf_ahead, const __grid_constant__ CUtensorMap map, int bk, bool pairs)
@@ -297,8 +305,21 @@ k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __res
         return;
     }
     const int o1 = flat_row1(d.nkb), nk = kBlockCols * d.nkb;
+    if constexpr (V == kRowTwo) {
+        float2* Y = X + padded_len(N);
+        const float2* z = run_plan<false, 0>(p, FlatLd<0>{X}, Y, X);
+        if (bk > 0) {
+            float2* f = align128(z == X ? Y : X);
+            separate_flat<0>(z, N, d.nh, nk, o1, f, row_max_threads(V));
+            if (threadIdx.x == 0) tma_store_pair(d, &map, f, o1, bk, r0, has1, blockIdx.y);
+        } else {
+            store_pair_spectra<true>(d, z, N, r0, has1, shat);
+        }
+        return;
+    }
+    if constexpr (V == kRow6000) pairs = PAIRS;
     float2* f = align128(X);
-    run_row_forward<V>(p, X, bk > 0 && pairs, f, o1);
+    run_row_forward<V>(p, X, pairs, f, o1);
     if (bk > 0) {
         if (pairs) {
             for (int k = d.nh + threadIdx.x; k < nk; k += blockDim.x) f[k] = f[o1 + k] = make_float2(0.f, 0.f);
@@ -306,7 +327,8 @@ k_rows_r2c_direct(ConvDims d, FftPlan p, float* __restrict__ grid, float2* __res
             __syncthreads();
         } else {
             // frequencies per thread: a runtime plan's block holds at least n / 32 threads
-            separate_flat<17>(X, N, d.nh, nk, o1, f);
+            separate_flat<V == kRow6000 ? 12 : 17>(X, N, d.nh, nk, o1, f,
+                                                   V == kRow6000 ? row_max_threads(V) : blockDim.x);
         }
         if (threadIdx.x == 0) tma_store_pair(d, &map, f, o1, bk, r0, has1, blockIdx.y);
         return;
@@ -334,13 +356,15 @@ k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
     stage_herm_pair(mt, mt, w0, has1 ? w0 + 1 : w0, has1, d.n_w, d.nh, p.n, X, d.noise_amp,
                     d.noise_seed + (uint64_t)waves.ev[blockIdx.y], d.plane_id);
     __syncthreads();
-    run_row_inverse<V>(p, X);
+    constexpr bool PAD = V == kRowTwo;
     const float2* z = X;
+    if constexpr (V == kRowTwo) z = run_plan<true, 0>(p, FlatLd<0>{X}, X + padded_len(p.n), X);
+    else run_row_inverse<V>(p, X);
     if (d.adc_max > 0) {                       // digitized: uint16 codes at the same rows
         uint16_t* adc = reinterpret_cast<uint16_t*>(wave);
         uint16_t* a0 = adc + (int64_t)w0 * d.n_t;
         const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(adc) & 3) == 0);
-        store_real_pair_adc(z, a0, a0 + d.n_t, d.n_t, has1, vec, d.adc_gain, d.adc_pedestal,
+        store_real_pair_adc<PAD>(z, a0, a0 + d.n_t, d.n_t, has1, vec, d.adc_gain, d.adc_pedestal,
                             (float)d.adc_max);
         return;
     }
@@ -349,7 +373,7 @@ k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
         const float* t0 = d.target + (int64_t)w0 * d.n_t;
         const bool vec = ((d.n_t & 1) == 0) &&
                          (((reinterpret_cast<uintptr_t>(wave) | reinterpret_cast<uintptr_t>(d.target)) & 7) == 0);
-        float ss = store_residual_pair(z, o0, o0 + d.n_t, t0, t0 + d.n_t, d.n_t, has1, vec);
+        float ss = store_residual_pair<PAD>(z, o0, o0 + d.n_t, t0, t0 + d.n_t, d.n_t, has1, vec);
         if (d.loss) {                          // one FP64 addition per warp (no static
 #pragma unroll                                         // shared memory: see attrs())
             for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -358,7 +382,7 @@ k_rows_c2r(ConvDims d, FftPlan p, const float2* __restrict__ mt, WavePtrs waves)
         return;
     }
     const bool vec = ((d.n_t & 1) == 0) && ((reinterpret_cast<uintptr_t>(wave) & 7) == 0);
-    store_real_pair(z, o0, o0 + d.n_t, d.n_t, has1, vec);
+    store_real_pair<PAD>(z, o0, o0 + d.n_t, d.n_t, has1, vec);
 }
 
 // CTAs of the direct R2C kernel k resident on the whole GPU with smem bytes each, when its
@@ -406,14 +430,39 @@ cudaError_t attrs()
         if (!e) e = cudaFuncSetAttribute(WCSIM_ROW_KERNEL(k_rows_c2r, v),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     }
+    if (!e) e = cudaFuncSetAttribute(k_rows_r2c_direct<kRow6000, false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     if (!e) g_attr.mark();
     return e;
+}
+
+// One launch of the direct R2C kernel over n_ev events.
+cudaError_t launch_direct(const ConvDims& d, const FftPlan& pt, float* grid, float2* shat, int n_ev,
+                          const ConvDims* like, cudaStream_t s)
+{
+    const int64_t n_pairs = ((int64_t)d.n_w * d.n_imp + 1) / 2;
+    CUtensorMap map;
+    int bk = r2c_store_map(d, pt, shat, n_ev, &map);
+    RowLaunch l = row_launch(pt, n_pairs * n_ev, kRowForward, bk > 0);
+    if (like && l.variant != kRow6000) {
+        l = row_launch(pt, ((int64_t)like->n_w * like->n_imp + 1) / 2, kRowForward, bk > 0);
+        if (l.variant != kRowTwo) {
+            bk = 0;
+            l.threads = row_block(pt, n_pairs);
+        }
+    }
+    if (like) l.pairs = false;
+    auto k = l.variant == kRow6000 && !l.pairs ? k_rows_r2c_direct<kRow6000, false>
+                                               : WCSIM_ROW_KERNEL(k_rows_r2c_direct, l.variant);
+    return launch_chained(d.chained != 0, k, dim3((unsigned)n_pairs, (unsigned)n_ev), l.threads, l.smem,
+                          s, d, pt, grid, shat, r2c_prefetch_ahead(d, grid, k, l.threads, l.smem), map,
+                          bk, l.pairs);
 }
 
 }  // namespace
 
 cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* grid,
-                            float2* shat, int* flags, cudaStream_t s, bool pairs)
+                            float2* shat, int* flags, cudaStream_t s, const ConvDims* like)
 {
     cudaError_t e = attrs();
     if (e) return e;
@@ -426,15 +475,7 @@ cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* g
         k_rows_r2c_staged<<<grid_n, kStagedThreads, smem, s>>>(d, pt, grid, shat, flags);
     } else {
         // the kernel writes the grid only with d.clear_input (consume and clear)
-        const int t = row_block(pt, n_pairs);
-        auto k = WCSIM_ROW_KERNEL(k_rows_r2c_direct, row_variant(pt, t));
-        const size_t sm = row_plan_smem(pt);
-        CUtensorMap map;
-        const int bk = r2c_store_map(d, pt, shat, 1, &map);
-        return launch_chained(d.chained != 0, k, (unsigned)n_pairs, t, sm, s, d, pt,
-                              const_cast<float*>(grid), shat,
-                              r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
-                              pairs && row_pairs(pt, pt.npass - 1));
+        return launch_direct(d, pt, const_cast<float*>(grid), shat, 1, like, s);
     }
     return cudaGetLastError();
 }
@@ -454,27 +495,16 @@ cudaError_t launch_rows_c2r_batch(const ConvDims& d, const FftPlan& pt, const fl
     cudaError_t e = attrs();
     if (e) return e;
     const dim3 grid((unsigned)((d.n_w + 1) / 2), (unsigned)n_ev);
-    const int t = row_block(pt, (int64_t)grid.x * grid.y);
-    auto k = WCSIM_ROW_KERNEL(k_rows_c2r, row_variant(pt, t));
-    return launch_chained(d.chained != 0, k, grid, t, row_plan_smem(pt), s, d, pt, mt, waves);
+    const RowLaunch l = row_launch(pt, (int64_t)grid.x * grid.y, kRowFrame, false);
+    auto k = WCSIM_ROW_KERNEL(k_rows_c2r, l.variant);
+    return launch_chained(d.chained != 0, k, grid, l.threads, l.smem, s, d, pt, mt, waves);
 }
 
 cudaError_t launch_rows_r2c_batch(const ConvDims& d, const FftPlan& pt, const float* grid,
                                   float2* shat, int n_ev, cudaStream_t s)
 {
-    constexpr bool pairs = true;
-    cudaError_t e = attrs();
-    if (e) return e;
-    const int64_t n_pairs = ((int64_t)d.n_w * d.n_imp + 1) / 2;
-    const dim3 g((unsigned)n_pairs, (unsigned)n_ev);
-    const int t = row_block(pt, n_pairs * n_ev);
-    auto k = WCSIM_ROW_KERNEL(k_rows_r2c_direct, row_variant(pt, t));
-    const size_t sm = row_plan_smem(pt);
-    CUtensorMap map;
-    const int bk = r2c_store_map(d, pt, shat, n_ev, &map);
-    return launch_chained(d.chained != 0, k, g, t, sm, s, d, pt, const_cast<float*>(grid), shat,
-                          r2c_prefetch_ahead(d, grid, k, t, sm), map, bk,
-                          pairs && row_pairs(pt, pt.npass - 1));
+    const cudaError_t e = attrs();
+    return e ? e : launch_direct(d, pt, const_cast<float*>(grid), shat, n_ev, nullptr, s);
 }
 
 }  // namespace wcsim

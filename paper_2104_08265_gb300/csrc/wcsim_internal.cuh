@@ -189,11 +189,14 @@ __host__ __device__ inline int64_t blk_index(int kt, int w, int n)
 cudaError_t launch_make_hermitian(const ConvDims& d, const float2* resp, float2* H, float scale,
                                   cudaStream_t s);
 // Time-axis real-to-complex FFT of every grid row; writes Shat_j blocked
-// [n_imp][nkb][n_w][4].  pairs = false: the last pass takes its butterflies one by one (a fit's
-// gradients are sums of both signs over the whole frame, and the transform of dL/dM keeps the
-// arithmetic whose rounding errors differ between the two halves of each pair).
+// [n_imp][nkb][n_w][4].  like: the transform of dL/dM, in the kernel instance that S's transform with
+// the dims *like takes (an adjoint has just run it, or will find it no colder than another), with the
+// last pass's butterflies one by one (a fit's gradients are sums of both signs over the whole frame,
+// and the transform of dL/dM keeps the arithmetic whose rounding errors differ between the two halves
+// of each pair).
 cudaError_t launch_rows_r2c(const ConvDims& d, const FftPlan& pt, const float* grid,
-                            float2* shat, int* flags, cudaStream_t s, bool pairs = true);
+                            float2* shat, int* flags, cudaStream_t s,
+                            const ConvDims* like = nullptr);
 // Same for n_ev events laid out with the ConvDims event strides (direct kernel).
 cudaError_t launch_rows_r2c_batch(const ConvDims& d, const FftPlan& pt, const float* grid,
                                   float2* shat, int n_ev, cudaStream_t s);
