@@ -238,8 +238,9 @@ wcsim_status wcsim_plane_set_forward(wcsim_plane* plane, int32_t fused);
 /* Rasterization tile of this plane (the autotuner's first choice, settable by hand; without
  * either, each call takes one by its number of depos): depos_per_block depos per 256 threads,
  * each rasterized by lanes_per_depo lanes.
- * Supported: (32, 8), (64, 8), (128, 8), (256, 8), (64, 16), (128, 16), (256, 16),
- * (64, 32), (128, 32), (256, 32); WCSIM_EINVAL otherwise.  Results are unchanged up to summation order.
+ * Supported: (32, 8), (64, 8), (128, 8), (256, 8), (16, 16), (64, 16), (128, 16), (256, 16),
+ * (8, 32), (64, 32), (128, 32), (256, 32), which holds every tile that the autotuner reports;
+ * WCSIM_EINVAL otherwise.  Results are unchanged up to summation order.
  * Host-only. */
 wcsim_status wcsim_plane_set_raster_tile(wcsim_plane* plane, int32_t depos_per_block,
                                          int32_t lanes_per_depo);

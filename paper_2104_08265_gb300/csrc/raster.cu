@@ -719,13 +719,17 @@ __global__ void k_windows(RasterConsts c, DepoArrays d, int32_t* __restrict__ ou
 // lanes per depo.
 bool raster_tile_supported(int depos_per_block, int lanes_per_depo)
 {
-    const int lo = lanes_per_depo == 8 ? 32 : 64;
     if (lanes_per_depo != 8 && lanes_per_depo != 16 && lanes_per_depo != 32) return false;
+    // 4 depos per warp at least, 8 with more lanes each; and raster_tile's own for the exact binomial
+    const int lo = lanes_per_depo == 8 ? 32 : 64;
+    if ((depos_per_block == 8 && lanes_per_depo == 32) || (depos_per_block == 16 && lanes_per_depo == 16)) return true;
     return depos_per_block >= lo && depos_per_block <= 256 && (depos_per_block & (depos_per_block - 1)) == 0;
 }
 
 RasterTile raster_tile(const RasterConsts& c, int64_t n_depos)
 {
+    // (so many depos that a launch of fewer per warp would have too many blocks)
+    if (n_depos > (1ll << 30)) return {16, 8};
     if (c.depos_per_block > 0) return {c.depos_per_block / 8, c.lanes_per_depo};
     // One depo per warp for the exact binomial's long serial walks, two above 64k depos (2000
     // depos: 76 us against 210 with 4 x 8 lanes; 30k: 418 / 472; 100k: 1234 with 2 x 16, 1275 with
