@@ -731,14 +731,15 @@ RasterTile raster_tile(const RasterConsts& c, int64_t n_depos)
     // (so many depos that a launch of fewer per warp would have too many blocks)
     if (n_depos > (1ll << 30)) return {16, 8};
     if (c.depos_per_block > 0) return {c.depos_per_block / 8, c.lanes_per_depo};
-    // One depo per warp for the exact binomial's long serial walks, two above 64k depos (2000
-    // depos: 76 us against 210 with 4 x 8 lanes; 30k: 418 / 472; 100k: 1234 with 2 x 16, 1275 with
-    // 1 x 32, 1256 with 4 x 8), four above 256k (300k: 3654 against 3666 with 2 x 16).  Else 8 lanes per depo, and more depos per warp (fewer, better
-    // filled decisions) as soon as there are warps enough for every SM (with fluctuation, 4 / 8 /
-    // 16 depos per warp: 2000 depos 10.9 / 15 / 21 us, 30k 25.2 / 25.3 / 29, 100k 58.5 / 56.0 /
-    // 58.0, 300k 148 / 132 / 128, 1M 466 / 404 / 378; 32 is slower throughout).
-    if (c.fluctuate == 2)
-        return n_depos > 262144 ? RasterTile{4, 8} : n_depos > 65536 ? RasterTile{2, 16} : RasterTile{1, 32};
+    // One depo per warp for the exact binomial's long serial walks (2000 depos: 76 us against 210 with
+    // 4 x 8 lanes), two above 64k depos.  Along tracks, 1 x 32 / 2 x 16 / 4 x 8: 100k 1301 / 1231 / 1266
+    // us, 300k 3699 / 3408 / 3371; strewn evenly 1272 / 1524 / 1826 and 3734 / 4410 / 5148, so that more
+    // than two never pay.
+    if (c.fluctuate == 2) return n_depos > 65536 ? RasterTile{2, 16} : RasterTile{1, 32};
+    // Else 8 lanes per depo, and more depos per warp (fewer, better filled decisions) as soon as there
+    // are warps enough for every SM (with fluctuation, 4 / 8 / 16 depos per warp: 2000 depos 10.9 / 15 /
+    // 21 us, 30k 25.2 / 25.3 / 29, 100k 58.5 / 56.0 / 58.0, 300k 148 / 132 / 128, 1M 466 / 404 / 378; 32
+    // is slower throughout).
     return {n_depos > 196608 ? 16 : n_depos > 40000 ? 8 : 4, 8};
 }
 
