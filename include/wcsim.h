@@ -259,7 +259,7 @@ typedef struct {
 } wcsim_tune_report;
 
 /* Time the kernel variants of this plane on `depos` (DEVICE) and keep the fastest: the
- * rasterization tile (depos per CTA, lanes per depo), the radices and order of the time-axis FFT plan (the cheapest
+ * rasterization tile (depos per 256 threads, lanes per depo), the radices and order of the time-axis FFT plan (the cheapest
  * plans with the fewest passes), the time-axis forward kernel, the wire-pass kernel and the
  * forward variant (plain or fused, wcsim_plane_set_forward).
  * Results are unchanged up to floating-point rounding order.  Synchronizes `stream`,

@@ -13,7 +13,7 @@
 // WCSIM_ROWS_KERNEL) is persistent: one CTA per SM walks pairs of rows, and one bulk copy
 // brings both rows of the next pair into a two-stage shared buffer while the previous pair
 // is transformed.  The inverse kernel stages its Hermitian input (each element read once,
-// its mirror written from the same load) and writes 4 ticks per 16-byte store, or, given a
+// its mirror written from the same load) and writes 2 ticks per 8-byte store, or, given a
 // target frame, the residual M - target and its sum of squares.
 #include <cuda.h>
 #include <cuda_runtime.h>

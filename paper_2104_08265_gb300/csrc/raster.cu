@@ -5,9 +5,10 @@
 // Work split.  A warp owns a run of consecutive depos (4 to 32, chosen by the number of depos).
 // Its lanes take the bin decision of one depo each and park what the rasterization needs of it in
 // shared memory; then each group of 8 lanes takes the warp's depos one by one (the four groups of
-// a warp work on four depos side by side): its lanes compute one erfc per bin edge of the patch
-// (rows and ticks together), difference them into the per-bin 1D weights in shared memory and
-// stride over (row, 4-tick group) items.  Warps never wait for one another.
+// a warp work on four depos side by side): its lanes form the 1D weights of the patch (rows and ticks
+// together) in shared memory, each from a series about the bin's centre, or where bins are wide
+// against sigma from differences of one erfc per bin edge, and stride over (row, 4-tick group) items.
+// Warps never wait for one another.
 // An item draws one Philox block for its four ticks when fluctuating (four Box-Muller
 // normals), forms Q' w_p w_t per bin and adds the four values into the grid with one
 // vector reduction.  The exact binomial fluctuation (an instance of its own) strides over
@@ -505,10 +506,9 @@ __host__ __device__ constexpr int adjoint_warp_smem(int depos_per_warp)
 // t_a = t + t_d and sigma = sqrt(2 D t_d).  The global sums are reduced per block in FP64.
 // Bound by instructions: a block whose first two warps decided for eight, kept the edge terms in
 // shared memory (58 KB per block, three blocks per SM) and divided for every item's row took 70 us
-// on 100k depos of the 960 x 6000 plane, this 56 us (2000 depos 12.5 / 8.8 us).  Depos per warp:
-// as the rasterizer, 16 above 64k depos, 8, 4 below 16k.  The order of every sum over a patch is
-// as it was: the per-depo results keep
-// their bits.
+// on 100k depos of the 960 x 6000 plane, this 56 us (2000 depos 12.5 / 8.8 us).  Depos per warp: 16
+// above 64k depos, 8 above 16k, else 4.  The order of every sum over a patch is as it was: the per-depo
+// results keep their bits.
 template <bool RN>
 __global__ void __launch_bounds__(kRasterWarps * 32, 8)
 k_depo_adjoint(RasterConsts c, DepoArrays d, const float* __restrict__ dgrid, DepoGrads g,

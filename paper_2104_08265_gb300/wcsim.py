@@ -413,7 +413,7 @@ class Plane:
         check(lib().wcsim_plane_set_forward(self._h, 1 if fused else 0))
 
     def set_raster_tile(self, depos_per_block: int, lanes_per_depo: int):
-        """Rasterization tile (depos per CTA, lanes per depo); see
+        """Rasterization tile (depos per 256 threads, lanes per depo); see
         wcsim_plane_set_raster_tile."""
         check(lib().wcsim_plane_set_raster_tile(self._h, int(depos_per_block),
                                                 int(lanes_per_depo)))
