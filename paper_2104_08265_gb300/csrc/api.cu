@@ -491,29 +491,29 @@ wcsim_status prepare_group(wcsim_plane* pl, int k, int32_t* clean_after, cudaStr
     return WCSIM_OK;
 }
 
-// The per-plane rasterization of events idx[0..k) (when the batch's one launch does not
-// apply) into their grid slots.
-wcsim_status rasterize_group(wcsim_plane* pl, int k, const int32_t* idx, const wcsim_depos* depos,
-                             cudaStream_t s)
+// One rasterization of events idx[0..k) of a batch (idx null: the first k) into their planes' batch
+// grids, slot[e] of event e, with the tile of the first one's plane.
+wcsim_status rasterize_events(wcsim_plane* const* planes, int k, const int32_t* idx,
+                              const int32_t* slot, const wcsim_depos* depos, cudaStream_t s)
 {
-    const ConvDims& d0 = pl->dims;
-    RasterConsts c = make_consts(pl);
-    BatchEvents ev;
-    ev.n = k;
-    ev.block_start[0] = 0;
+    BatchPlanes q;
     int64_t total = 0;
-    for (int i = 0; i < k; ++i) total += depos[idx[i]].n;
-    const RasterTile tile = raster_tile(c, total);
+    for (int i = 0; i < k; ++i) total += depos[idx ? idx[i] : i].n;
+    const RasterTile tile = raster_tile(make_consts(planes[idx ? idx[0] : 0]), total);
+    q.n = k;
+    q.block_start[0] = 0;
     for (int i = 0; i < k; ++i) {
-        const wcsim_depos* dp = &depos[idx[i]];
-        ev.d[i] = depo_arrays(dp);
-        ev.grid[i] = pl->bgrid + (size_t)i * ev_grid_elems(d0);
-        const uint64_t seed = pl->prm.seed + (uint64_t)idx[i];     // per-event stream
-        ev.key0[i] = (uint32_t)seed;
-        ev.key1[i] = (uint32_t)(seed >> 32);
-        ev.block_start[i + 1] = ev.block_start[i] + rasterize_blocks(dp->n, tile.depos_per_warp);
+        const int e = idx ? idx[i] : i;
+        wcsim_plane* p = planes[e];
+        q.c[i] = make_consts(p);
+        const uint64_t seed = p->prm.seed + (uint64_t)e;         // per-event stream
+        q.c[i].keys.set((uint32_t)seed, (uint32_t)(seed >> 32));
+        q.d[i] = depo_arrays(&depos[e]);
+        q.grid[i] = p->bgrid + (size_t)slot[e] * ev_grid_elems(p->dims);
+        q.flags[i] = p->flags;
+        q.block_start[i + 1] = q.block_start[i] + rasterize_blocks(depos[e].n, tile.depos_per_warp);
     }
-    cudaError_t e = launch_rasterize_batch(c, ev, tile, pl->flags, s);
+    const cudaError_t e = launch_rasterize_events(q, tile, s);
     return e ? cuda_fail(e, "batch rasterize launch") : WCSIM_OK;
 }
 
@@ -996,27 +996,11 @@ wcsim_status wcsim_batch_run(int32_t n_events, wcsim_plane* const* planes,
                    (p->prm.fluctuate == 2) == (c0.fluctuate == 2);
     }
     if (together) {
-        BatchPlanes q;
-        int64_t n_depos = 0;
-        for (int i = 0; i < n_events; ++i) n_depos += depos[i].n;
-        const RasterTile tile = raster_tile(c0, n_depos);
-        q.n = n_events;
-        q.block_start[0] = 0;
-        for (int i = 0; i < n_events; ++i) {
-            wcsim_plane* p = planes[i];
-            q.c[i] = make_consts(p);
-            const uint64_t seed = p->prm.seed + (uint64_t)i;         // per-event stream
-            q.c[i].keys.set((uint32_t)seed, (uint32_t)(seed >> 32));
-            q.d[i] = depo_arrays(&depos[i]);
-            q.grid[i] = p->bgrid + (size_t)slot[i] * ev_grid_elems(p->dims);
-            q.flags[i] = p->flags;
-            q.block_start[i + 1] = q.block_start[i] + rasterize_blocks(depos[i].n, tile.depos_per_warp);
-        }
-        cudaError_t e = launch_rasterize_events(q, tile, s);
-        if (e) return cuda_fail(e, "batch rasterize launch");
+        wcsim_status st = rasterize_events(planes, n_events, nullptr, slot, depos, s);
+        if (st) return st;
     } else {
         for (int g = 0; g < n_groups; ++g) {
-            wcsim_status st = rasterize_group(planes[first[g]], count[g], members[g], depos, s);
+            wcsim_status st = rasterize_events(planes, count[g], members[g], slot, depos, s);
             if (st) return st;
         }
     }

@@ -394,23 +394,6 @@ k_rasterize(RasterConsts c, DepoArrays d, float* __restrict__ grid, int* flags, 
                             smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
 }
 
-// Several events of one plane: CTA b belongs to the event whose block range holds b.
-template <int G, int MODE>
-__global__ void __launch_bounds__(kRasterWarps * 32)
-k_rasterize_batch(RasterConsts c, BatchEvents ev, int* flags, int dpw)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ float s_stirl[MODE == 2 ? 16 : 1];
-    load_stirling<MODE>(c, s_stirl);
-    const int warp = threadIdx.x >> 5;
-    int e = 0;
-    while (e + 1 < ev.n && ev.block_start[e + 1] <= (int)blockIdx.x) ++e;
-    c.keys.set(ev.key0[e], ev.key1[e]);
-    rasterize_warp<G, MODE>(c, ev.d[e], ev.grid[e], flags,
-                            (((int64_t)blockIdx.x - ev.block_start[e]) * kRasterWarps + warp) * dpw, dpw,
-                            smraw + warp * raster_warp_smem(MODE, dpw, G), s_stirl);
-}
-
 // Every event of a batch in one launch, each with its plane's own constants.  A warp's share of depos
 // is a piece, a block's worth of pieces one item of block_start, in the events' order.  The constants
 // are read through the event's index, and a round key that the compiler then holds costs a register:
@@ -783,17 +766,6 @@ cudaError_t launch_rasterize(const RasterConsts& c, const DepoArrays& d, float* 
         return launch_chained(c.chained != 0, k, blocks, kRasterWarps * 32, smem, s, c, d, grid,
                               flags, t.depos_per_warp));
     return cudaSuccess;
-}
-
-cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
-                                   const RasterTile& t, int* flags, cudaStream_t s)
-{
-    const int blocks = ev.block_start[ev.n];
-    if (blocks <= 0) return cudaSuccess;
-    const int smem = kRasterWarps * raster_warp_smem(c.fluctuate, t.depos_per_warp, t.lanes_per_depo);
-    WCSIM_RASTER_DISPATCH(k_rasterize_batch, t.lanes_per_depo, c.fluctuate,
-        k<<<blocks, kRasterWarps * 32, smem, s>>>(c, ev, flags, t.depos_per_warp));
-    return cudaGetLastError();
 }
 
 cudaError_t launch_rasterize_events(const BatchPlanes& q, const RasterTile& t, cudaStream_t s)

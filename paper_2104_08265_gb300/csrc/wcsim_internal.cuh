@@ -51,15 +51,6 @@ struct DepoArrays {
 
 constexpr int kMaxBatch = 64;          // events per batched launch
 
-// Per-event inputs of a batched rasterization, passed by value.
-struct BatchEvents {
-    int32_t n;
-    int32_t block_start[kMaxBatch + 1];  // first CTA of each event (prefix sum)
-    DepoArrays d[kMaxBatch];
-    float* grid[kMaxBatch];
-    uint32_t key0[kMaxBatch], key1[kMaxBatch];
-};
-
 // Every event of a batch, whatever its plane, for one rasterization; passed by value.
 struct BatchPlanes {
     int32_t n;
@@ -85,9 +76,6 @@ struct RasterTile {
 };
 // The plane's tile if one was set, else the rule by the number of depos and fluctuation mode.
 RasterTile raster_tile(const RasterConsts& c, int64_t n_depos);
-// Rasterize several events of one plane in one launch (c.keys ignored: per event).
-cudaError_t launch_rasterize_batch(const RasterConsts& c, const BatchEvents& ev,
-                                   const RasterTile& t, int* flags, cudaStream_t s);
 // CTAs that n_depos depos take.
 int rasterize_blocks(int64_t n_depos, int depos_per_warp);
 // Rasterize every event of q in one launch with the tile t.  Events with the normal fluctuation and
