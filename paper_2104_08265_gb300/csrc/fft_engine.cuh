@@ -843,8 +843,8 @@ __host__ inline int row_threads(const FftPlan& p)
 // two buffers (run_plan, 256 threads).  The in-place ones keep 72 (448) to 80 registers per thread, so
 // that registers and shared memory give out together: 24 warps per SM at 6000 points, 26 at 9600,
 // where two buffers leave 8 to 16.  What they pay for it is code: every pass unrolls the butterflies
-// that a thread holds (the runtime ones spill 48 to 124 bytes per thread, that of 448 threads 192 to
-// 792), and a kernel of one wave or two spends much of its time fetching instructions.
+// that a thread holds (the runtime ones spill 48 to 200 bytes per thread, that of 448 threads 192 to
+// 836), and a kernel of one wave or two spends much of its time fetching instructions.
 enum RowVariant : int { kRow6000 = 0, kRow384, kRow448, kRow704, kRowTwo, kRowVariants };
 __host__ __device__ constexpr int row_max_threads(int v)
 {
