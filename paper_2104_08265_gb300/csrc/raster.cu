@@ -720,15 +720,15 @@ RasterTile raster_tile(const RasterConsts& c, int64_t n_depos)
     // than two never pay.
     if (c.fluctuate == 2) return n_depos > 65536 ? RasterTile{2, 16} : RasterTile{1, 32};
     // Else 8 lanes per depo, and more depos per warp (fewer, better filled decisions) as soon as there
-    // are warps enough for every SM (with fluctuation, 4 / 8 / 16 depos per warp: 2000 depos 7.6 / 10.8 /
-    // 17.2 us, 20k 18.7 / 18.0 / 22.0, 30k 24.3 / 24.4 / 26.1, 100k 58.5 / 56.0 / 58.0, 300k 148 / 132 /
-    // 128, 1M 466 / 404 / 378; 32 is slower throughout).
-    // Four up to 16k depos: depos that reach few bins are mostly decision (30k points 10.3 / 7.9 us, 7.4
-    // before the warps decided for themselves).  Rows that are not 16-byte aligned take scalar additions,
-    // whose patches last longer: four up to 40k, never 16 (5999 ticks, mean path: 40k 27.4 / 31.0 us, 200k
-    // 159 / 161 / 165).
+    // are warps enough for every SM.  With fluctuation, 4 / 8 / 16 depos per warp: 2000 depos 7.6 / 10.8 /
+    // 17.2 us, 10k along tracks 7.9 / 8.3 / 10.8, 12.5k 9.2 / 8.3 / 11.5, 30k 24.3 / 24.4 / 26.1, 100k 58.5 /
+    // 56.0 / 58.0, 300k 148 / 132 / 128, 1M 466 / 404 / 378; 32 is slower throughout.  On the mean path, and
+    // where depos reach few bins, the decision is more of the work (5000 depos along tracks 5.0 / 5.2 us, 8000
+    // 5.9 / 5.6, 12.5k 7.5 / 6.2, before the warps decided for themselves 6.5; 30k points 10.3 / 7.9, 7.4).
+    // Rows that are not 16-byte aligned take scalar additions, whose patches last longer: four up to 40k,
+    // never 16 (5999 ticks, mean path: 40k 27.4 / 31.0 us, 200k 159 / 161 / 165).
     if ((c.n_ticks & 3) != 0) return {n_depos > 40000 ? 8 : 4, 8};
-    return {n_depos > 196608 ? 16 : n_depos > 16384 ? 8 : 4, 8};
+    return {n_depos > 196608 ? 16 : n_depos > (c.fluctuate ? 11000 : 7000) ? 8 : 4, 8};
 }
 
 int rasterize_blocks(int64_t n_depos, int depos_per_warp)
