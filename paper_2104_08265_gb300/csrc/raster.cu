@@ -724,10 +724,9 @@ RasterTile raster_tile(const RasterConsts& c, int64_t n_depos)
     // 17.2 us, 10k along tracks 7.9 / 8.3 / 10.8, 12.5k 9.2 / 8.3 / 11.5, 30k 24.3 / 24.4 / 26.1, 100k 58.5 /
     // 56.0 / 58.0, 300k 148 / 132 / 128, 1M 466 / 404 / 378; 32 is slower throughout.  On the mean path, and
     // where depos reach few bins, the decision is more of the work (5000 depos along tracks 5.0 / 5.2 us, 8000
-    // 5.9 / 5.6, 12.5k 7.5 / 6.2, before the warps decided for themselves 6.5; 30k points 10.3 / 7.9, 7.4).
-    // Rows that are not 16-byte aligned take scalar additions, whose patches last longer: four up to 40k,
-    // never 16 (5999 ticks, mean path: 40k 27.4 / 31.0 us, 200k 159 / 161 / 165).
-    if ((c.n_ticks & 3) != 0) return {n_depos > 40000 ? 8 : 4, 8};
+    // 5.9 / 5.6, 12.5k 7.5 / 6.2, before the warps decided for themselves 6.5; 30k points 10.3 / 7.9, 7.4).  Rows that are not 16-byte
+    // aligned, whose patches are added bin by bin, behave alike along tracks (5998 ticks: 12.5k 14.3 / 12.6 /
+    // 15.5, 250k 195 / 172 / 159), and are nearly indifferent for evenly strewn depos (200k 159 / 161 / 165).
     return {n_depos > 196608 ? 16 : n_depos > (c.fluctuate ? 11000 : 7000) ? 8 : 4, 8};
 }
 
